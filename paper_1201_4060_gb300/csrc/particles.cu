@@ -173,7 +173,8 @@ __device__ __forceinline__ unsigned warp_inclusive(unsigned v, unsigned lane) {
 template <bool SPLIT>
 __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__ count, unsigned* __restrict__ offset,
                                                     unsigned* __restrict__ cursor, unsigned* __restrict__ chunk,
-                                                    unsigned* __restrict__ item, unsigned NB, unsigned below) {
+                                                    unsigned* __restrict__ item, unsigned NB, unsigned below,
+                                                    unsigned chunk_len) {
     __shared__ unsigned wd[32], wsp[32], wc[32], s_total;
     const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // total of the dense bricks (the start of the sparse range)
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
         const unsigned ci = i < NB ? count[i] : 0u;
         const bool dense = !SPLIT || ci >= below;
         const unsigned vd0 = dense ? ci : 0u, vs0 = dense ? 0u : ci;
-        const unsigned nc = dense ? (ci + kChunk - 1) / kChunk : 0u;
+        const unsigned nc = dense ? (ci + chunk_len - 1) / chunk_len : 0u;
         const unsigned vd = warp_inclusive(vd0, lane), vc = warp_inclusive(nc, lane);
         const unsigned vs = SPLIT ? warp_inclusive(vs0, lane) : 0u;
         if (lane == 31) {
@@ -371,10 +372,11 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    const size_t need = carve<TR>(&w, nullptr, NB, P);
+    const unsigned len = item_particles(p->dtype, P, NB);
+    const size_t need = carve<TR>(&w, nullptr, NB, P, len);
     int rc = p->pws.grow(need);
     if (rc) return rc;
-    carve<TR>(&w, p->pws.ptr, NB, P);
+    carve<TR>(&w, p->pws.ptr, NB, P, len);
     const cudaStream_t main_stream = p->stream;
     cudaStream_t st = sort_stream ? sort_stream : main_stream;
     p->stream = st;                                     // stage timers follow the sort's stream
@@ -410,8 +412,8 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        if (below > 0) scan_kernel<true><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below);
-        else scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u);
+        if (below > 0) scan_kernel<true><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below, len);
+        else scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -447,7 +449,8 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    carve<TR>(&w, ws, NB, P);
+    const unsigned len = item_particles(p->dtype, P, NB);
+    carve<TR>(&w, ws, NB, P, len);
     cudaStream_t st = p->stream;
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (NB + 2), st)) != cudaSuccess) return set_cuda_error(e);
@@ -456,7 +459,7 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const bool grad = !(flags & BSPLINE_INTERP_NO_GRAD);
     bin_kernel<TR, false, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, status,
                                                                NB < kAggregateBricks, (AT*)nullptr, (AT*)nullptr);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u);
+    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len);
     scatter_kernel<TR, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, (AT*)out_u, grad ? (AT*)out_grad : nullptr,
                                                              NB < kAggregateBricks, status);
     int rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
@@ -513,7 +516,7 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u);
+        scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -560,7 +563,7 @@ int run_sort_order(bspline_plan_s* p, const double* x, int64_t P, int* perm) {
     const int agg = NB < kAggregateBricks;
     bin_kernel<TR, false, float><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, p->d_status, agg,
                                                                    (float*)nullptr, (float*)nullptr);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u);
+    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk);
     scatter_kernel<TR, float, false, true><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w,
                                                                             (float*)nullptr, (float*)nullptr, agg,
                                                                             p->d_status, perm);
@@ -605,10 +608,10 @@ size_t interp_workspace_bytes(const bspline_plan_s* p, int64_t P) {
     const unsigned NB = g.NB;
     if (p->dtype == BSPLINE_F64) {
         Ws<double> w;
-        return carve<double>(&w, nullptr, NB, P);
+        return carve<double>(&w, nullptr, NB, P, item_particles(p->dtype, P, NB));
     }
     Ws<float> w;
-    return carve<float>(&w, nullptr, NB, P);
+    return carve<float>(&w, nullptr, NB, P, item_particles(p->dtype, P, NB));
 }
 
 int launch_interp_split(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u,

@@ -7,6 +7,7 @@
 
 #include <cstring>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace bs {
@@ -42,6 +43,12 @@ static_assert(sizeof(Rec<float>) == 32 && sizeof(Rec<double>) == 32, "one sector
 // Particles per gather work item: a brick with more particles is split into
 // several items, each staging the brick's tile, so no CTA serialises a clump.
 constexpr unsigned kChunk = 2048;
+// FP64 plans' evaluation: 512, and 42 when the bricks hold few particles (three components of 42 particles
+// are the 126 units of a 128-thread CTA; gather_fixed).
+constexpr unsigned kFixedLong = 512, kFixedShort = 42;
+inline unsigned item_particles(int dtype, int64_t P, unsigned NB) {
+    return dtype != BSPLINE_F64 ? kChunk : (P >= 256LL * NB ? kFixedLong : kFixedShort);
+}
 
 template <typename TR> struct Ws {
     unsigned* count;    // [NB + 2]  particles per brick; slot NB = invalid positions; NB + 1 = *unsorted
@@ -49,13 +56,13 @@ template <typename TR> struct Ws {
     unsigned* offset;   // [NB + 3]  start of each brick's sorted segment; [NB] end of the valid
                         //           particles, [NB + 1] end of all, [NB + 2] start of the sparse range
     unsigned* cursor;   // [NB + 1]  next free sorted slot of each brick (starts at offset)
-    unsigned* chunk;    // [NB + 1]  exclusive prefix sum of ceil(count / kChunk): first work item of a brick
-    unsigned* item;     // [NB + ceil(P / kChunk)]  brick of each work item (the first chunk[NB] are set)
+    unsigned* chunk;    // [NB + 1]  exclusive prefix sum of ceil(count / chunk_len): first work item of a brick
+    unsigned* item;     // [NB + ceil(P / chunk_len)]  brick of each work item (the first chunk[NB] are set)
     long long P;        // particles
     Rec<TR>* s_rec;     // [P]       located records sorted by brick
 };
 
-inline size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
+constexpr size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
 template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t P, unsigned chunk_len = kChunk) {
     size_t off = 0;
@@ -601,59 +608,11 @@ __device__ __forceinline__ void stage_brick(typename TileT<CT>::T* tile, const C
     stage_tile<ORD, CT, BYO>(tile, coef, N, x0, y0, z0);
 }
 
-// u and grad u of one particle from the staged tile (Table 1 contraction,
-// z axis first).  base points at the particle's first stencil node.
-template <int ORD, typename A, bool GRAD, int SX, int SY, int TS>
-__device__ __forceinline__ void eval_particle(const A* __restrict__ base, A tx, A ty, A tz, A dscale,
-                                              A* __restrict__ out_u, A* __restrict__ out_grad) {
-    A wx[ORD], dwx[ORD], wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
-    bspline_weights<ORD, A>(tx, wx, dwx);
-    bspline_weights<ORD, A>(ty, wy, dwy);
-    bspline_weights<ORD, A>(tz, wz, dwz);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const A* tc = base + c * TS;
-        A u = 0, gx = 0, gy = 0, gz = 0;
-#pragma unroll
-        for (int jx = 0; jx < ORD; ++jx) {
-            A y00 = 0, y10 = 0, y01 = 0;
-#pragma unroll
-            for (int jy = 0; jy < ORD; ++jy) {
-                const A* line = tc + jx * SX + jy * SY;
-                A z0v = 0, z1v = 0;
-#pragma unroll
-                for (int jz = 0; jz < ORD; ++jz) {
-                    const A a = line[jz];
-                    z0v = fma(wz[jz], a, z0v);
-                    if (GRAD) z1v = fma(dwz[jz], a, z1v);
-                }
-                y00 = fma(wy[jy], z0v, y00);
-                if (GRAD) {
-                    y10 = fma(dwy[jy], z0v, y10);
-                    y01 = fma(wy[jy], z1v, y01);
-                }
-            }
-            u = fma(wx[jx], y00, u);
-            if (GRAD) {
-                gx = fma(dwx[jx], y00, gx);
-                gy = fma(wx[jx], y10, gy);
-                gz = fma(wx[jx], y01, gz);
-            }
-        }
-        out_u[c] = u;
-        if (GRAD) {
-            out_grad[3 * c + 0] = gx * dscale;
-            out_grad[3 * c + 1] = gy * dscale;
-            out_grad[3 * c + 2] = gz * dscale;
-        }
-    }
-}
-
 // Packed two-way FP32 contraction (fma.rn.f32x2) of one component:
 // adjacent y-lines jy, jy + 1 are contracted along z together (their loads
 // form the pair, the z weight is duplicated), and their y-sums are kept as
-// (even, odd) pairs that are added at the end of each x-plane.  Same
-// arithmetic per term as eval_particle; the sums are grouped by parity of jy.
+// (even, odd) pairs that are added at the end of each x-plane.  The
+// sums are grouped by parity of jy.
 // ld(jx, jy, jz) gives the coefficient at stencil node (jx, jy, jz): the
 // staged gather reads its shared-memory tile, the direct gather global
 // memory, with the same arithmetic in the same order, so the two agree bit
@@ -868,40 +827,221 @@ __device__ __forceinline__ void eval_bf16(const unsigned* __restrict__ base, int
     }
 }
 
-// FP64: one thread per particle (the FP64 pipe, not shared memory, bounds it).
-template <int ORD, typename TR, bool GRAD>
-__global__ void __launch_bounds__(128)
-gather_f64(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, double* __restrict__ out_u,
-           double* __restrict__ out_grad, double dscale, unsigned long long* __restrict__ status) {
+// u and grad u of one component of one particle in FP64 arithmetic, its stencil read from global memory
+// (comp: the component's [N][N][N] coefficients; a: the first stencil node).  The evaluation of the few
+// particles whose stencil the fixed-point form below does not represent: never inlined, rolled loops.
+template <int ORD, bool GRAD>
+__device__ __noinline__ void eval_f64_global(const double* __restrict__ comp, int N, int ax, int ay, int az, double tx,
+                                             double ty, double tz, double dscale, double* out) {
+    double wx[ORD], dwx[ORD], wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
+    bspline_weights<ORD, double>(tx, wx, dwx);
+    bspline_weights<ORD, double>(ty, wy, dwy);
+    bspline_weights<ORD, double>(tz, wz, dwz);
+    double u = 0, gx = 0, gy = 0, gz = 0;
+#pragma unroll 1
+    for (int jx = 0; jx < ORD; ++jx) {
+        double y00 = 0, y10 = 0, y01 = 0;
+#pragma unroll 1
+        for (int jy = 0; jy < ORD; ++jy) {
+            const double* line = comp + ((size_t)wrap_index(ax + jx, N) * N + wrap_index(ay + jy, N)) * N;
+            double z0 = 0, z1 = 0;
+#pragma unroll 1
+            for (int jz = 0; jz < ORD; ++jz) {
+                const double v = line[wrap_index(az + jz, N)];
+                z0 = fma(wz[jz], v, z0);
+                if (GRAD) z1 = fma(dwz[jz], v, z1);
+            }
+            y00 = fma(wy[jy], z0, y00);
+            if (GRAD) {
+                y10 = fma(dwy[jy], z0, y10);
+                y01 = fma(wy[jy], z1, y01);
+            }
+        }
+        u = fma(wx[jx], y00, u);
+        if (GRAD) {
+            gx = fma(dwx[jx], y00, gx);
+            gy = fma(wx[jx], y10, gy);
+            gz = fma(wx[jx], y01, gz);
+        }
+    }
+    out[0] = u;
+    if (GRAD) {
+        out[1] = gx * dscale;
+        out[2] = gy * dscale;
+        out[3] = gz * dscale;
+    }
+}
+
+// FP64 plans: one CTA per work item, the brick's coefficients staged and turned into 60-bit fixed point
+// (fixed.cuh) at one scale per component, the largest magnitude in the tile; weights, contraction and
+// derivatives are integer multiply-adds, and only the twelve results are FP64 again.  Bound: integer issue.
+// The FP64 pipe took 1900 operations a particle at order 6: 5.36 ms for 10^6 particles on 256^3; the fixed
+// form's 5100 wide multiply-adds, with the tile's conversion (216 values a particle there), take 1.72 ms.
+// A stencil value is rounded at 2^-60 of the tile's largest, so the result is
+// at least as accurate as FP64 arithmetic (2^-53) for a stencil whose own largest value is within 2^kSpare
+// of the tile's; the others, and every particle of a component whose tile holds a NaN or an infinity or
+// nothing above 2^-895, are evaluated in FP64 from global memory (eval_f64_global).  That choice depends on the coefficients and the position
+// alone, so every route to the evaluation gives the same bits.
+// NC = 3: a thread takes a particle's components in turn; NC = 1 (items of up to 42 particles): a thread
+// takes one component of a particle, the axes' weights being shared: with the 30 particles a brick of the
+// case above three of the four warps would idle otherwise (2.99 ms).
+constexpr int kSpare = 6;
+template <int ORD, int NC> constexpr int fixed_threads() { return NC == 3 && ORD >= 7 ? 192 : 128; }
+template <int ORD, typename TR, bool GRAD, int NC>
+__global__ void __launch_bounds__(fixed_threads<ORD, NC>(), ORD >= 7 ? 2 : (ORD <= 4 ? 4 : 3))
+gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, unsigned chunk_len,
+             double* __restrict__ out_u, double* __restrict__ out_grad, double dscale,
+             unsigned long long* __restrict__ status) {
     using S = Shape<double, ORD>;
+    constexpr int T = fixed_threads<ORD, NC>();
+    if (blockIdx.x >= w.chunk[bg.NB]) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* tile = reinterpret_cast<double*>(smem_raw);
-    const unsigned brick = blockIdx.x;
-    const unsigned beg = w.offset[brick], end = beg + w.count[brick];
-    if (beg == end) return;
+    __shared__ unsigned s_top[3], s_any[3];
+    const unsigned brick = w.item[blockIdx.x];
+    const unsigned beg = w.offset[brick] + (blockIdx.x - w.chunk[brick]) * chunk_len;
+    const unsigned n = min(chunk_len, w.offset[brick] + w.count[brick] - beg);
     int x0, y0, z0;
     brick_origin<S::BX, S::BY, S::BZ>(brick, bg, &x0, &y0, &z0);
-    stage_brick<ORD, double>(tile, coef, N, x0, y0, z0);
+    // the tile, 16 lanes a z-row
+    static_assert(S::EZ <= 16 && T % 16 == 0 && T / 16 <= 2 * S::EY, "16 lanes a row");
+    uint2* words = reinterpret_cast<uint2*>(smem_raw);
+    {
+        const int z = threadIdx.x & 15;
+        int ix = 0, iy = threadIdx.x >> 4;
+        const double* col = coef + wrap_index(z0 + z, N);
+        for (int r = iy; r < S::EX * S::EY; r += T / 16) {
+            while (iy >= S::EY) {
+                iy -= S::EY;
+                ++ix;
+            }
+            const double* src = col + ((size_t)wrap_index(x0 + ix, N) * N + wrap_index(y0 + iy, N)) * N;
+            if (z < S::EZ) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) cp_async8(words + c * S::TS + r * S::PZ + z, src + (size_t)c * N * N * N);
+            }
+            iy += T / 16;
+        }
+    }
+    if (threadIdx.x < 3) s_top[threadIdx.x] = s_any[threadIdx.x] = 0;
     cp_async_wait_all();
     __syncthreads();
-    for (unsigned i = beg + threadIdx.x; i < end; i += blockDim.x) {
-        const Rec<TR> rc = w.s_rec[i];
-        const int ox = (int)(rc.cell >> (2 * kAnchorBits)) - x0;
-        const int oy = (int)((rc.cell >> kAnchorBits) & 1023u) - y0;
+    // each component's largest high word and any bit but signs
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+        unsigned top = 0, any = 0;
+        for (int k = threadIdx.x; k < S::TS; k += T) {
+            const uint2 d = words[c * S::TS + k];
+            top = max(top, d.y & 0x7fffffffu);
+            any |= d.x;
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        any = __reduce_or_sync(0xffffffffu, any) | top;
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&s_top[c], top);
+            atomicOr(&s_any[c], any);
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+        const int emax = (int)(s_top[c] >> 20);
+        for (int k = threadIdx.x; k < S::TS; k += T) {
+            const uint2 d = words[c * S::TS + k];
+            const fixed::Limbs l = fixed::limbs(fixed::from_double(d.y, d.x, emax));
+            words[c * S::TS + k] = make_uint2((unsigned)l.lo, (unsigned)l.hi);
+        }
+    }
+    __syncthreads();
+    int4* ws = reinterpret_cast<int4*>(smem_raw + align_up(tile_bytes<ORD, double>()));
+    // components c0 .. c0 + NC - 1 of one particle; wx(j): the x weights of node j
+    auto evaluate = [&](const Rec<TR>& rc, int c0, auto wx, const fixed::Limbs (&wy)[ORD], const fixed::Limbs (&dwy)[ORD],
+                        const fixed::Limbs (&wz)[ORD], const fixed::Limbs (&dwz)[ORD]) {
+        const int ax = (int)(rc.cell >> (2 * kAnchorBits)), ay = (int)((rc.cell >> kAnchorBits) & 1023u);
+        const int az = (int)(rc.cell & 1023u);
+        const size_t idx = rc.idx;
+        const uint2* base = words + (ax - x0) * S::SX + (ay - y0) * S::SY + (az - z0);
+        unsigned left = 0;                               // components that the fixed form does not represent
+#pragma unroll 1
+        for (int c = c0; c < c0 + NC; ++c) {
+            long long f[4];
+            int size = 0;
+            const uint2* tc = base + c * S::TS;
+            fixed::contract<ORD, GRAD>(
+                [&](int jx, int jy, int jz) {
+                    const uint2 v = tc[jx * S::SX + jy * S::SY + jz];
+                    return fixed::Limbs{(int)v.y, (int)v.x};
+                },
+                wx, wy, dwy, wz, dwz, f, &size);
+            const int emax = (int)(s_top[c] >> 20);
+            if (!s_any[c]) f[0] = f[1] = f[2] = f[3] = 0;            // a component that is zero in the whole tile
+            else if (emax < fixed::kMinExponent || emax == 2047 || size < (1 << (29 - kSpare))) left |= 1u << c;
+            // V 2^(emax - 1081), in two exact steps (one of them may leave the normal range)
+            const int k = emax - 1081, k1 = k / 2;
+            const double s1 = __hiloint2double((1023 + k1) << 20, 0), s2 = __hiloint2double((1023 + k - k1) << 20, 0);
+            out_u[3 * idx + c] = ((double)f[0] * s1) * s2;
+            if (GRAD) {
+#pragma unroll
+                for (int e = 0; e < 3; ++e) out_grad[9 * idx + 3 * c + e] = (((double)f[1 + e] * s1) * s2) * dscale;
+            }
+        }
+        if (left) {
+#pragma unroll 1
+            for (int c = 0; c < 3; ++c) {
+                if (!(left >> c & 1u)) continue;
+                double r[4];
+                eval_f64_global<ORD, GRAD>(coef + (size_t)c * N * N * N, N, ax, ay, az, rc.t[0], rc.t[1], rc.t[2],
+                                           dscale, r);
+                out_u[3 * idx + c] = r[0];
+                if (GRAD) {
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) out_grad[9 * idx + 3 * c + e] = r[1 + e];
+                }
+            }
+        }
+    };
+    auto record_ok = [&](const Rec<TR>& rc) {
+        const int ox = (int)(rc.cell >> (2 * kAnchorBits)) - x0, oy = (int)((rc.cell >> kAnchorBits) & 1023u) - y0;
         const int oz = (int)(rc.cell & 1023u) - z0;
-        const unsigned idx = rc.idx;
-        if (!BS_CHECK_OK(ox >= 0 && ox < S::BX && oy >= 0 && oy < S::BY && oz >= 0 && oz < S::BZ &&
-                             (long long)idx < w.P,
-                         status + kStatusBounds))
-            continue;
-        double u[3], gr[9];
-        eval_particle<ORD, double, GRAD, S::SX, S::SY, S::TS>(tile + ox * S::SX + oy * S::SY + oz, (double)rc.t[0],
-                                                               (double)rc.t[1], (double)rc.t[2], dscale, u, gr);
+        return BS_CHECK_OK(ox >= 0 && ox < S::BX && oy >= 0 && oy < S::BY && oz >= 0 && oz < S::BZ &&
+                               (long long)rc.idx < w.P,
+                           status + kStatusBounds);
+    };
+    const auto fixed_t = [](double t) { return __double2ll_rn(t * 1152921504606846976.0); };     // t 2^60
+    fixed::Limbs wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
+    if constexpr (NC == 1) {
+        // thread (a, q): the weights of particle q along axis a, then its component a
+        const unsigned a = threadIdx.x / n, q = threadIdx.x - a * n;
+        const bool on = threadIdx.x < 3 * n;
+        Rec<TR> rc;
+        if (on) {
+            rc = w.s_rec[beg + q];
+            fixed::weights<ORD>(fixed_t(a == 0 ? rc.t[0] : (a == 1 ? rc.t[1] : rc.t[2])), wy, dwy);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) out_u[3 * (size_t)idx + c] = u[c];
-        if (GRAD) {
+            for (int j = 0; j < ORD; ++j)
+                ws[(a * ORD + j) * kFixedShort + q] = make_int4(wy[j].hi, wy[j].lo, dwy[j].hi, dwy[j].lo);
+        }
+        __syncthreads();
+        if (!on || !record_ok(rc)) return;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) out_grad[9 * (size_t)idx + k] = gr[k];
+        for (int j = 0; j < ORD; ++j) {
+            const int4 y = ws[(ORD + j) * kFixedShort + q], v = ws[(2 * ORD + j) * kFixedShort + q];
+            wy[j] = {y.x, y.y};
+            dwy[j] = {y.z, y.w};
+            wz[j] = {v.x, v.y};
+            dwz[j] = {v.z, v.w};
+        }
+        evaluate(rc, (int)a, [&](int j) { return ws[j * kFixedShort + q]; }, wy, dwy, wz, dwz);
+    } else {
+        for (unsigned i = threadIdx.x; i < n; i += T) {
+            const Rec<TR> rc = w.s_rec[beg + i];
+            if (!record_ok(rc)) continue;
+            fixed::weights<ORD>(fixed_t(rc.t[0]), wy, dwy);
+#pragma unroll
+            for (int j = 0; j < ORD; ++j)                // the x weights wait in shared memory
+                ws[j * T + threadIdx.x] = make_int4(wy[j].hi, wy[j].lo, dwy[j].hi, dwy[j].lo);
+            fixed::weights<ORD>(fixed_t(rc.t[1]), wy, dwy);
+            fixed::weights<ORD>(fixed_t(rc.t[2]), wz, dwz);
+            evaluate(rc, 0, [&](int j) { return ws[j * T + threadIdx.x]; }, wy, dwy, wz, dwz);
         }
     }
 }
@@ -1233,10 +1373,18 @@ int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, voi
     const AT dscale = (AT)((double)p->N / p->L);
     int rc;
     if constexpr (sizeof(AT) == 8) {
-        auto k = grad ? gather_f64<ORD, TR, true> : gather_f64<ORD, TR, false>;
-        if ((rc = set_smem(k, sm))) return rc;
-        k<<<NB, 128, sm, p->stream>>>(reinterpret_cast<const double*>(coeffs), p->N, g, w, (double*)out_u,
-                                      grad ? (double*)out_grad : nullptr, dscale, p->d_status);
+        const unsigned len = item_particles(p->dtype, w.P, NB);
+        const bool whole = len == kFixedLong;
+        auto k = whole ? (grad ? gather_fixed<ORD, TR, true, 3> : gather_fixed<ORD, TR, false, 3>)
+                       : (grad ? gather_fixed<ORD, TR, true, 1> : gather_fixed<ORD, TR, false, 1>);
+        const int threads = whole ? fixed_threads<ORD, 3>() : fixed_threads<ORD, 1>();
+        // the tile and the weights of the particles in work
+        const size_t sm_x = align_up(sm) + sizeof(int4) * ORD * (whole ? threads : 3 * kFixedShort);
+        if ((rc = set_smem(k, sm_x))) return rc;
+        const long long items = (long long)NB + (w.P + len - 1) / len;
+        k<<<(unsigned)items, threads, sm_x, p->stream>>>(
+            reinterpret_cast<const double*>(coeffs), p->N, g, w, len, (double*)out_u, grad ? (double*)out_grad : nullptr,
+            dscale, p->d_status);
     } else {
         auto k = grad ? gather_f32<ORD, CT, TR, true> : gather_f32<ORD, CT, TR, false>;
         // room to align the tile to 128 bytes; BF16: the two copies of the pair tile
