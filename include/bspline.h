@@ -134,15 +134,18 @@ int bspline_plan_set_stream(bspline_plan_t plan, void* stream);
 
 /* Gather split.  Particles are sorted by brick; a brick holding fewer than
  * direct_below particles is evaluated by the direct gather (each particle's
- * stencil read from global memory, a thread per particle), the others by the
+ * stencil read from global memory), the others by the
  * staged gather (the brick's coefficient tile staged in shared memory, a CTA
  * per up to 2048 of its particles).  Both give the same results bit for bit;
  * only the time differs: a staged brick carries a fixed cost of a few
  * microseconds of dependent latency, which a handful of particles does not
  * repay.  0 stages every brick.  FP32 and BF16 plans (FP64 plans always
- * stage).  BSPLINE_GATHER_SPLIT_AUTO (the default) takes 32 for a call with
- * fewer than 12 particles per brick on average and 0 otherwise;
- * bspline_plan_autotune picks the split by timing. */
+ * stage).  BSPLINE_GATHER_SPLIT_AUTO (the default) takes 4096 / n^3 for a call
+ * with fewer than that many particles per brick on average and 0 otherwise;
+ * bspline_plan_autotune picks the split by timing.  With AUTO and with "every
+ * brick direct" (0xffffffff) a call of at most 12 Mi / n^3 particles (without
+ * BSPLINE_INTERP_SORTED) is not sorted at all: the direct gather takes the
+ * particles in the caller's order, without workspace. */
 #define BSPLINE_GATHER_SPLIT_AUTO 0xfffffffeu
 int bspline_plan_set_gather_split(bspline_plan_t plan, unsigned direct_below);
 

@@ -153,9 +153,10 @@ __global__ void bin_kernel(const double* __restrict__ x, long long P, int N, dou
 // Places the bricks' segments in the sorted order and counts the staged
 // gather's work items.  Bricks holding at least `below` particles ("dense":
 // every brick when below = 0) come first, in brick order; the bricks below
-// it ("sparse", evaluated by the direct gather) follow, in brick order, so
-// the direct gather runs flat over one contiguous range; the invalid bin NB
-// comes last.  Writes offset[b] (and its copy cursor[b] for the placement
+// it ("sparse", evaluated by the direct gather) follow, placed from the end
+// of the valid particles downwards (so that no pass has to total the dense
+// ones first), and the direct gather runs flat over one contiguous range; the
+// invalid bin NB comes last.  Writes offset[b] (and its copy cursor[b] for the placement
 // pass), offset[NB] = the end of the valid particles, offset[NB + 1] = the
 // end of all, offset[NB + 2] = the start of the sparse range; chunk[] (dense
 // bricks only) the exclusive prefix sum of the work items, ceil(count /
@@ -170,41 +171,51 @@ __device__ __forceinline__ unsigned warp_inclusive(unsigned v, unsigned lane) {
 }
 
 // SPLIT = false (below = 0: every brick dense) skips the sparse bookkeeping.
+// Bound: one CTA's latency per tile.  A thread takes kScanRun consecutive bricks (16-byte loads and
+// stores), the next tile's counts requested before this tile is scanned: 44032 bricks (512^3) in 6 tiles
+// instead of 43.
+constexpr unsigned kScanRun = 8;
 template <bool SPLIT>
 __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__ count, unsigned* __restrict__ offset,
                                                     unsigned* __restrict__ cursor, unsigned* __restrict__ chunk,
                                                     unsigned* __restrict__ item, unsigned NB, unsigned below,
-                                                    unsigned chunk_len) {
-    __shared__ unsigned wd[32], wsp[32], wc[32], s_total;
+                                                    unsigned chunk_len, long long P) {
+    __shared__ unsigned wd[32], wsp[32], wc[32];
     const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    // total of the dense bricks (the start of the sparse range)
-    unsigned D = 0;
-    if constexpr (SPLIT) {
-        unsigned dsum = 0;
-        for (unsigned i = t; i < NB; i += 1024) {
-            const unsigned ci = count[i];
-            if (ci >= below) dsum += ci;
+    const unsigned V = (unsigned)P - count[NB];           // valid particles
+    unsigned v[kScanRun], nx[kScanRun];
+    auto load = [&](unsigned b0) {                        // the run's counts, zero beyond the bricks
+        const unsigned i = b0 + t * kScanRun;
+        if (i + kScanRun <= NB) {
+#pragma unroll
+            for (unsigned k = 0; k < kScanRun; k += 4) {
+                const uint4 q = *reinterpret_cast<const uint4*>(count + i + k);
+                nx[k] = q.x;
+                nx[k + 1] = q.y;
+                nx[k + 2] = q.z;
+                nx[k + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (unsigned k = 0; k < kScanRun; ++k) nx[k] = i + k < NB ? count[i + k] : 0u;
         }
-        dsum = __reduce_add_sync(0xffffffffu, dsum);
-        if (lane == 0) wd[warp] = dsum;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned v = __reduce_add_sync(0xffffffffu, wd[lane]);
-            if (lane == 0) s_total = v;
-        }
-        __syncthreads();
-        D = s_total;
-    }
+    };
     unsigned cd = 0, cs = 0, cc = 0;                      // carries: dense, sparse, items
-    // tiles of 1024 consecutive bricks, one per thread: warp scans, then a scan of the 32 warp totals
-    for (unsigned b0 = 0; b0 < NB; b0 += 1024) {
-        const unsigned i = b0 + t;
-        const unsigned ci = i < NB ? count[i] : 0u;
-        const bool dense = !SPLIT || ci >= below;
-        const unsigned vd0 = dense ? ci : 0u, vs0 = dense ? 0u : ci;
-        const unsigned nc = dense ? (ci + chunk_len - 1) / chunk_len : 0u;
-        const unsigned vd = warp_inclusive(vd0, lane), vc = warp_inclusive(nc, lane);
-        const unsigned vs = SPLIT ? warp_inclusive(vs0, lane) : 0u;
+    // tiles of 1024 runs: sums of the runs, warp scans of those, then a scan of the 32 warp totals
+    load(0);
+    for (unsigned b0 = 0; b0 < NB; b0 += 1024 * kScanRun) {
+        unsigned sd = 0, ss = 0, sc = 0;
+#pragma unroll
+        for (unsigned k = 0; k < kScanRun; ++k) {
+            v[k] = nx[k];
+            const bool dense = !SPLIT || v[k] >= below;
+            sd += dense ? v[k] : 0u;
+            ss += dense ? 0u : v[k];
+            sc += dense ? (v[k] + chunk_len - 1) / chunk_len : 0u;
+        }
+        if (b0 + 1024 * kScanRun < NB) load(b0 + 1024 * kScanRun);
+        const unsigned vd = warp_inclusive(sd, lane), vc = warp_inclusive(sc, lane);
+        const unsigned vs = SPLIT ? warp_inclusive(ss, lane) : 0u;
         if (lane == 31) {
             wd[warp] = vd;
             wsp[warp] = vs;
@@ -217,15 +228,38 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
             wc[lane] = warp_inclusive(wc[lane], lane);
         }
         __syncthreads();
-        const unsigned exd = cd + (warp ? wd[warp - 1] : 0u) + vd - vd0;          // exclusive
-        const unsigned exs = cs + (warp ? wsp[warp - 1] : 0u) + vs - vs0;
-        const unsigned exc = cc + (warp ? wc[warp - 1] : 0u) + vc - nc;
-        if (i < NB) {
-            const unsigned o = dense ? exd : D + exs;
-            offset[i] = o;
-            cursor[i] = o;
-            chunk[i] = exc;
-            for (unsigned k = 0; k < nc; ++k) item[exc + k] = i;
+        unsigned exd = cd + (warp ? wd[warp - 1] : 0u) + vd - sd;                 // exclusive
+        unsigned exs = V - cs - (warp ? wsp[warp - 1] : 0u) - vs + ss;              // end of the run's segments
+        unsigned exc = cc + (warp ? wc[warp - 1] : 0u) + vc - sc;
+        const unsigned i = b0 + t * kScanRun;
+        unsigned o[kScanRun], c[kScanRun];
+#pragma unroll
+        for (unsigned k = 0; k < kScanRun; ++k) {
+            const bool dense = !SPLIT || v[k] >= below;
+            exs -= dense ? 0u : v[k];
+            o[k] = dense ? exd : exs;
+            c[k] = exc;
+            const unsigned nc = dense ? (v[k] + chunk_len - 1) / chunk_len : 0u;
+            for (unsigned q = 0; q < nc; ++q) item[exc + q] = i + k;
+            exd += dense ? v[k] : 0u;
+            exc += nc;
+        }
+        if (i + kScanRun <= NB) {
+#pragma unroll
+            for (unsigned k = 0; k < kScanRun; k += 4) {
+                const uint4 a = make_uint4(o[k], o[k + 1], o[k + 2], o[k + 3]);
+                *reinterpret_cast<uint4*>(offset + i + k) = a;
+                *reinterpret_cast<uint4*>(cursor + i + k) = a;
+                *reinterpret_cast<uint4*>(chunk + i + k) = make_uint4(c[k], c[k + 1], c[k + 2], c[k + 3]);
+            }
+        } else {
+#pragma unroll
+            for (unsigned k = 0; k < kScanRun; ++k)
+                if (i + k < NB) {
+                    offset[i + k] = o[k];
+                    cursor[i + k] = o[k];
+                    chunk[i + k] = c[k];
+                }
         }
         cd += wd[31];
         cs += wsp[31];
@@ -233,10 +267,10 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
         __syncthreads();                                  // the totals are read before the next tile
     }
     if (t == 0) {
-        offset[NB] = cd + cs;                             // the invalid bin
-        cursor[NB] = cd + cs;
-        offset[NB + 1] = cd + cs + count[NB];
-        offset[NB + 2] = SPLIT ? D : cd;
+        offset[NB] = V;                                   // the invalid bin
+        cursor[NB] = V;
+        offset[NB + 1] = (unsigned)P;
+        offset[NB + 2] = cd;
         chunk[NB] = cc;
     }
 }
@@ -330,30 +364,30 @@ __global__ void scatter_kernel(const double* __restrict__ x, long long P, int N,
 
 template <typename CT, typename AT, typename TR>
 int dispatch_order(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, void* out_u,
-                   void* out_grad, bool grad) {
+                   void* out_grad, bool grad, unsigned below) {
     switch (p->order) {
-        case 2: return run_gather<2, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 3: return run_gather<3, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 4: return run_gather<4, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 5: return run_gather<5, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 6: return run_gather<6, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 7: return run_gather<7, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
-        case 8: return run_gather<8, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
+        case 2: return run_gather<2, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 3: return run_gather<3, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 4: return run_gather<4, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 5: return run_gather<5, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 6: return run_gather<6, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 7: return run_gather<7, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 8: return run_gather<8, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
     }
     return BSPLINE_ERR_UNSUPPORTED_ORDER;
 }
 
 template <typename CT, typename AT, typename TR>
-int dispatch_direct(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, void* out_u, void* out_grad,
-                    bool grad, unsigned below) {
+int dispatch_points(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, Ws<TR> w, unsigned NB,
+                    void* out_u, void* out_grad, bool grad) {
     switch (p->order) {
-        case 2: return run_gather_direct<2, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 3: return run_gather_direct<3, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 4: return run_gather_direct<4, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 5: return run_gather_direct<5, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 6: return run_gather_direct<6, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 7: return run_gather_direct<7, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
-        case 8: return run_gather_direct<8, CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        case 2: return run_gather_points<2, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 3: return run_gather_points<3, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 4: return run_gather_points<4, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 5: return run_gather_points<5, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 6: return run_gather_points<6, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 7: return run_gather_points<7, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
+        case 8: return run_gather_points<8, CT, AT, TR>(p, coeffs, x, P, w, NB, out_u, out_grad, grad);
     }
     return BSPLINE_ERR_UNSUPPORTED_ORDER;
 }
@@ -364,11 +398,53 @@ inline unsigned grid_for(long long P, int threads) {
     return (unsigned)(g < 1 ? 1 : g);
 }
 
+// Whether a call evaluates its particles in the caller's order, each straight from global memory
+// (gather_points), instead of sorting them.  The direct gather costs about 0.0035 n^3 ns a particle while
+// the coefficients stay in L2 and two to three times that beyond; the sorted calls cost 25 to 100 us of
+// launches and passes and then 0.3 ns a particle.  Measured (us, unsorted / sorted, FP32): 64^3 order 4,
+// 10^3 particles 13 / 26; 128^3 order 6, 16000 20 / 41, 64000 56 / 59, 256000 197 / 124; 256^3 order 4,
+// 64000 46 / 63, 256000 161 / 138; 512^3 order 6, 64000 157 / 179; 256^3 order 2, 10^6 161 / 224.
+constexpr long long kUnsortedNodes = 12LL << 20;        // particles times n^3
+bool unsorted_call(const bspline_plan_s* p, int64_t P, int flags) {
+    if (p->dtype == BSPLINE_F64 || (flags & BSPLINE_INTERP_SORTED)) return false;
+    if (p->direct_below != BSPLINE_GATHER_SPLIT_AUTO && p->direct_below != 0xffffffffu) return false;
+    return P * p->order * p->order * p->order <= kUnsortedNodes;
+}
+
+// The automatic split: a staged brick costs as much as about 4096 / n^3 particles of the direct gather; a
+// call whose bricks hold fewer than that on average is split there, a denser one is staged throughout.
+// Measured (us, every brick direct / staged, FP32): 512^3, 24 particles a brick: order 2 296 / 667, order 4
+// 481 / 763, order 6 956 / 888; 256^3, 45 a brick: order 3 100 / 130, order 4 129 / 138, order 6 268 / 171.
+unsigned auto_split(int64_t P, unsigned NB, int n) {
+    const unsigned below = 4096u / (unsigned)(n * n * n);
+    return P < (long long)below * NB ? below : 0u;
+}
+
+// The evaluation of such a call: the direct gather on the plan's stream, no workspace.
+template <typename CT, typename AT, typename TR>
+int run_points(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u, void* out_grad,
+               int flags) {
+    const cudaError_t e = cudaMemsetAsync(p->d_status, 0, sizeof(unsigned long long) * kStatusParticleWords, p->stream);
+    if (e != cudaSuccess) return set_cuda_error(e);
+    StageTimer tm(p, BSPLINE_STAGE_GATHER_DIRECT);
+    const int rc = dispatch_points<CT, AT, TR>(p, coeffs, x, P, Ws<TR>{}, 0u, out_u, out_grad,
+                                               !(flags & BSPLINE_INTERP_NO_GRAD));
+    return rc ? rc : set_cuda_error(cudaGetLastError());
+}
+
 // The sort (bin, scan, scatter) runs on sort_stream when one is given (it
 // needs only the positions) and the gather on the plan's stream after `sorted`.
 template <typename CT, typename AT, typename TR>
 int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u, void* out_grad,
                int flags, cudaStream_t sort_stream, cudaEvent_t sorted) {
+    if (unsorted_call(p, P, flags)) {
+        if (sort_stream) {                              // the positions may arrive on that stream
+            cudaError_t e = cudaEventRecord(sorted, sort_stream);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(p->stream, sorted, 0);
+            if (e != cudaSuccess) return set_cuda_error(e);
+        }
+        return run_points<CT, AT, TR>(p, coeffs, x, P, out_u, out_grad, flags);
+    }
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
@@ -402,7 +478,7 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     if (sort_stream && 2LL * p->sms < (long long)sort_grid) sort_grid = (unsigned)(2 * p->sms);
     // bricks with fewer particles than this go to the direct gather (FP32 accumulation only)
     unsigned below = p->direct_below;
-    if (below == BSPLINE_GATHER_SPLIT_AUTO) below = P < 12LL * NB ? 32u : 0u;
+    if (below == BSPLINE_GATHER_SPLIT_AUTO) below = auto_split(P, NB, p->order);
     if (sizeof(AT) == 8 || presorted) below = 0u;       // sorted input: bricks stay in input order
     const int agg = NB < kAggregateBricks || presorted;  // sorted input: a warp's particles share bricks
     {
@@ -412,8 +488,8 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        if (below > 0) scan_kernel<true><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below, len);
-        else scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len);
+        if (below > 0) scan_kernel<true><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below, len, P);
+        else scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len, P);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -430,12 +506,12 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     p->stream = main_stream;
     {
         StageTimer tm(p, BSPLINE_STAGE_GATHER);
-        rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
+        rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
     }
     if (rc) return rc;
     if (below > 0) {
         StageTimer tm(p, BSPLINE_STAGE_GATHER_DIRECT);
-        rc = dispatch_direct<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, below);
+        rc = dispatch_points<CT, AT, TR>(p, coeffs, nullptr, P, w, NB, out_u, out_grad, grad);
     }
     if (rc) return rc;
     return set_cuda_error(cudaGetLastError());
@@ -446,6 +522,7 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
 template <typename CT, typename AT, typename TR>
 int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const void* coeffs, const double* x,
                   int64_t P, void* out_u, void* out_grad, int flags) {
+    if (unsorted_call(p, P, flags)) return run_points<CT, AT, TR>(p, coeffs, x, P, out_u, out_grad, flags);
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
@@ -459,10 +536,10 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const bool grad = !(flags & BSPLINE_INTERP_NO_GRAD);
     bin_kernel<TR, false, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, status,
                                                                NB < kAggregateBricks, (AT*)nullptr, (AT*)nullptr);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len);
+    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len, P);
     scatter_kernel<TR, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, (AT*)out_u, grad ? (AT*)out_grad : nullptr,
                                                              NB < kAggregateBricks, status);
-    int rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad);
+    int rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, 0u);
     if (rc) return rc;
     return set_cuda_error(cudaGetLastError());
 }
@@ -516,7 +593,7 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk);
+        scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk, P);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -563,7 +640,7 @@ int run_sort_order(bspline_plan_s* p, const double* x, int64_t P, int* perm) {
     const int agg = NB < kAggregateBricks;
     bin_kernel<TR, false, float><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, p->d_status, agg,
                                                                    (float*)nullptr, (float*)nullptr);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk);
+    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk, P);
     scatter_kernel<TR, float, false, true><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w,
                                                                             (float*)nullptr, (float*)nullptr, agg,
                                                                             p->d_status, perm);
@@ -627,6 +704,8 @@ int launch_interp_split(bspline_plan_s* p, const void* coeffs, const double* x, 
     }
     return BSPLINE_ERR_INVALID_ARG;
 }
+
+bool interp_sorts(const bspline_plan_s* p, int64_t P, int flags) { return !unsorted_call(p, P, flags); }
 
 int launch_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u, void* out_grad,
                   int flags) {

@@ -141,6 +141,29 @@ __device__ __forceinline__ unsigned wrap_anchor(long long a, int N) {
     return (unsigned)(r < 0 ? r + N : r);
 }
 
+// One axis of Eq. alg-int-6: the first stencil node modulo N and t, from s = x N / L; false for a
+// non-finite s or one with no fractional bits left.
+template <typename TR>
+__device__ __forceinline__ bool locate_axis(double s, int N, int order, unsigned* anchor, TR* t) {
+    if constexpr (sizeof(TR) == 4) {
+        long long base;
+        if (locate_nonneg(s, order, &base, t)) {
+            *anchor = wrap_anchor(base + 1, N);
+            return true;
+        }
+    }
+    const double sh = s - 0.5 * order;
+    if (!(fabs(sh) < 4.0e15)) {          // NaN, Inf, or no fractional bits left
+        *anchor = 0;
+        *t = 0;
+        return false;
+    }
+    const double f = floor(sh);
+    *t = (TR)(sh - f);
+    *anchor = wrap_anchor((long long)f + 1, N);
+    return true;
+}
+
 // Locate one particle (Eq. alg-int-6): its brick key and record; the key is NB
 // for a non-finite position or one with no fractional bits left.
 template <typename TR>
@@ -151,28 +174,7 @@ __device__ __forceinline__ unsigned locate_particle(const double* __restrict__ x
     TR tt[3];
     bool ok = true;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double s = x[3 * p + a] * scale;
-        if constexpr (sizeof(TR) == 4) {
-            long long base;
-            float tf;
-            if (locate_nonneg(s, order, &base, &tf)) {
-                tt[a] = tf;
-                anc[a] = wrap_anchor(base + 1, N);
-                continue;
-            }
-        }
-        const double sh = s - 0.5 * order;
-        if (!(fabs(sh) < 4.0e15)) {      // NaN, Inf, or no fractional bits left
-            ok = false;
-            anc[a] = 0;
-            tt[a] = 0;
-            continue;
-        }
-        const double f = floor(sh);
-        tt[a] = (TR)(sh - f);
-        anc[a] = wrap_anchor((long long)f + 1, N);
-    }
+    for (int a = 0; a < 3; ++a) ok = locate_axis<TR>(x[3 * p + a] * scale, N, order, &anc[a], &tt[a]) && ok;
     if (!ok) return NB;
     r->cell = (anc[0] << (2 * kAnchorBits)) | (anc[1] << kAnchorBits) | anc[2];
     r->t[0] = tt[0];
@@ -1300,60 +1302,139 @@ gather_f32(const CT* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, float* __
                                        status);
 }
 
-// Direct gather for sparse bricks: the particles of bricks holding fewer
-// than the split (placed by the scan in one contiguous range after the dense
-// bricks, still grouped by brick) are evaluated straight from the
-// coefficient array, one thread per particle.  A staged work item costs a
-// few microseconds of dependent latency (records, bucketing, the tile copy)
-// whatever its particle count, so for a handful of particles reading the
-// stencils from global memory (through L1, where neighbouring threads'
-// particles share rows) is far cheaper.  Same contraction as the staged
-// gather (row_x2 / add_row in the same order), so the results are the same
-// bits.  The x-rows run in a rolled loop: unrolled, all 3 ORD^3 global loads
-// would be hoisted at once.
-template <int ORD, typename CT, typename TR, bool GRAD>
-__global__ void __launch_bounds__(256, 2)
-gather_direct(const CT* __restrict__ coef, int N, unsigned NB, Ws<TR> w, float* __restrict__ out_u,
-              float* __restrict__ out_grad, float dscale, unsigned long long* __restrict__ status) {
-    const unsigned beg = w.offset[NB + 2], end = w.offset[NB];
-    const size_t NN = (size_t)N * N;
-    for (unsigned i = beg + blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x) {
-        const Rec<TR> rc = w.s_rec[i];
-        const int ax = (int)(rc.cell >> (2 * kAnchorBits));
-        const int ay = (int)((rc.cell >> kAnchorBits) & 1023u);
-        const int az = (int)(rc.cell & 1023u);
-        if (!BS_CHECK_OK(ax < N && ay < N && az < N && (long long)rc.idx < w.P, status + kStatusBounds)) continue;
-        float wx[ORD], dwx[ORD], wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
-        bspline_weights<ORD, float>((float)rc.t[0], wx, dwx);
-        bspline_weights<ORD, float>((float)rc.t[1], wy, dwy);
-        bspline_weights<ORD, float>((float)rc.t[2], wz, dwz);
-        const PairWeights<ORD> pw(wz, dwz, wy, dwy);
-        int yo[ORD], zo[ORD];
+// Direct gather: particles evaluated from global memory, without a staged brick.  SORTED: those of the
+// bricks holding fewer than the split (placed by the scan in one contiguous range after the dense bricks);
+// otherwise every particle, in the caller's order, straight from its position (calls whose particles are
+// too few for a sort to pay: run_points).
+// A CTA takes G particles through four steps: thread (particle, axis) locates it and computes the axis'
+// weights; thread (particle, y-line, piece) copies the stencil lines' aligned 16-byte pieces to shared memory
+// (the pieces of a line are neighbouring threads', so a copy touches few cache lines, and a CTA's whole
+// input is in flight at once); thread (particle, component, x-row) contracts its row; thread (particle, component) adds the
+// rows up and stores.  Same contraction in the same order as the staged gather (row_x2, add_row), so the
+// results are the same bits.  Bound: DRAM sectors and latency; a thread per particle, which read each of its
+// 3 n^3 values through L1 by itself, cost 6 times as many L1 lookups.  Measured: 2^18 particles on 512^3, order 6, in brick order 386 -> 296 us;
+// 10^3 particles on 64^3, order 4, one launch instead of five, 35 -> 12 us a call.
+template <int ORD, typename CT> struct Points {
+    static constexpr int T = 128;
+    static constexpr int G = ORD == 8 ? 4 : T / (3 * ORD);   // particles of a CTA (order 8: 48 KB of shared memory)
+    static constexpr int V = 16 / (int)sizeof(CT);      // values of a piece
+    static constexpr int NQ = (ORD + 2 * V - 2) / V;    // pieces a line can touch
+    static constexpr int LINE = 4 * NQ;                 // words of a line
+    // words of an x-row; the skew spreads the rows' common offsets over the banks
+    static constexpr int ROW = ORD * LINE + ((ORD * LINE) % 8 == 0 ? 4 : 0);
+    static constexpr int WORDS = G * 3 * ORD * ROW;
+    static_assert(G * ORD * NQ <= T && G * 3 * ORD <= T, "one round of threads per step");
+};
+template <int ORD, typename CT, typename TR, bool GRAD, bool SORTED>
+__global__ void __launch_bounds__(Points<ORD, CT>::T)
+gather_points(const CT* __restrict__ coef, int N, const double* __restrict__ x, long long P, double scale, unsigned NB,
+              Ws<TR> w, float* __restrict__ out_u, float* __restrict__ out_grad, float dscale,
+              unsigned long long* __restrict__ status) {
+    using K = Points<ORD, CT>;
+    constexpr int T = K::T, G = K::G;
+    __shared__ __align__(16) unsigned s_line[K::WORDS];
+    __shared__ float s_w[G][3][2][ORD], s_sum[G][3 * ORD][3];
+    __shared__ int s_anchor[G][3];
+    __shared__ long long s_idx[G];
+    const long long beg = SORTED ? w.offset[NB + 2] : 0, end = SORTED ? w.offset[NB] : P;
+    const int tid = threadIdx.x;
+    for (long long i0 = beg + (long long)blockIdx.x * G; i0 < end; i0 += (long long)gridDim.x * G) {
+        if (tid < 3 * G) {
+            const int q = tid / 3, a = tid - 3 * q;
+            const long long i = i0 + q;
+            unsigned anchor = 0;
+            float t = 0.f;
+            bool ok = false;
+            if (i < end) {
+                if constexpr (SORTED) {
+                    const Rec<TR> rc = w.s_rec[i];
+                    anchor = (rc.cell >> (kAnchorBits * (2 - a))) & 1023u;
+                    t = a == 0 ? rc.t[0] : (a == 1 ? rc.t[1] : rc.t[2]);
+                    ok = BS_CHECK_OK((int)anchor < N && (long long)rc.idx < w.P, status + kStatusBounds);
+                    if (a == 0) s_idx[q] = rc.idx;
+                } else {
+                    ok = locate_axis<float>(x[3 * i + a] * scale, N, ORD, &anchor, &t);
+                    if (a == 0) s_idx[q] = i;
+                }
+            }
+            s_anchor[q][a] = ok ? (int)anchor : -1;
+            float wt[ORD], dwt[ORD];
+            bspline_weights<ORD, float>(t, wt, dwt);
 #pragma unroll
-        for (int j = 0; j < ORD; ++j) {
-            yo[j] = wrap_index(ay + j, N) * N;
-            zo[j] = wrap_index(az + j, N);
+            for (int j = 0; j < ORD; ++j) {
+                s_w[q][a][0][j] = wt[j];
+                s_w[q][a][1][j] = dwt[j];
+            }
         }
-        const size_t idx = rc.idx;
-#pragma unroll 1
-        for (int c = 0; c < 3; ++c) {
-            const CT* cb = coef + (size_t)c * N * NN;
-            float u = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll 1
-            for (int jx = 0; jx < ORD; ++jx) {
-                const CT* row = cb + (size_t)wrap_index(ax + jx, N) * NN;
+        __syncthreads();
+        const auto good = [&](int q) { return (s_anchor[q][0] | s_anchor[q][1] | s_anchor[q][2]) >= 0; };
+        // thread (particle, y-line, piece) copies that piece of every component and x-row: everything but the
+        // x index is the thread's own
+        if (tid < G * ORD * K::NQ) {
+            const int q = tid / (ORD * K::NQ), e = tid - q * (ORD * K::NQ), jy = e / K::NQ, k = e - jy * K::NQ;
+            const int ax = s_anchor[q][0], az = s_anchor[q][2];
+            if (good(q) && K::V * k < (az & (K::V - 1)) + ORD) {
+                const size_t NN = (size_t)N * N;
+                const CT* src = coef + (size_t)wrap_index(s_anchor[q][1] + jy, N) * N +
+                                wrap_index((az & ~(K::V - 1)) + K::V * k, N);
+                unsigned* dst = s_line + q * (3 * ORD) * K::ROW + jy * K::LINE + 4 * k;
+#pragma unroll
+                for (int jx = 0; jx < ORD; ++jx) {
+                    const CT* at = src + (size_t)wrap_index(ax + jx, N) * NN;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) cp_async16(dst + (c * ORD + jx) * K::ROW, at + (size_t)c * N * NN);
+                }
+            }
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        if (tid < G * 3 * ORD) {
+            const int q = tid / (3 * ORD), r = tid - q * 3 * ORD;
+            if (good(q)) {
+                float wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
+#pragma unroll
+                for (int j = 0; j < ORD; ++j) {
+                    wy[j] = s_w[q][1][0][j];
+                    dwy[j] = s_w[q][1][1][j];
+                    wz[j] = s_w[q][2][0][j];
+                    dwz[j] = s_w[q][2][1][j];
+                }
+                const PairWeights<ORD> pw(wz, dwz, wy, dwy);
+                const CT* line = reinterpret_cast<const CT*>(s_line + tid * K::ROW) + (s_anchor[q][2] & (K::V - 1));
                 float s00, s10, s01;
-                row_x2<ORD, GRAD>([&](int jy, int jz) { return widen<CT>(row[yo[jy] + zo[jz]]); }, pw, wy, dwy, wz, dwz,
-                                  &s00, &s10, &s01);
-                add_row<GRAD>(wx[jx], dwx[jx], s00, s10, s01, &u, &gx, &gy, &gz);
-            }
-            out_u[3 * idx + c] = u;
-            if (GRAD) {
-                out_grad[9 * idx + 3 * c + 0] = gx * dscale;
-                out_grad[9 * idx + 3 * c + 1] = gy * dscale;
-                out_grad[9 * idx + 3 * c + 2] = gz * dscale;
+                row_x2<ORD, GRAD>([&](int jy, int jz) { return widen<CT>(line[jy * K::NQ * K::V + jz]); }, pw, wy, dwy, wz,
+                                  dwz, &s00, &s10, &s01);
+                s_sum[q][r][0] = s00;
+                s_sum[q][r][1] = s10;
+                s_sum[q][r][2] = s01;
             }
         }
+        __syncthreads();
+        if (tid < 3 * G && i0 + tid / 3 < end) {
+            const int q = tid / 3, c = tid - 3 * q;
+            const size_t idx = (size_t)s_idx[q];
+            const bool ok = good(q);
+            float u = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+            if (ok) {
+#pragma unroll
+                for (int jx = 0; jx < ORD; ++jx) {
+                    const float* v = s_sum[q][c * ORD + jx];
+                    add_row<GRAD>(s_w[q][0][0][jx], s_w[q][0][1][jx], v[0], v[1], v[2], &u, &gx, &gy, &gz);
+                }
+            } else if (!SORTED) {
+                u = gx = gy = gz = NAN;
+                if (c == 0) atomicAdd(status + kStatusNonfinite, 1ULL);
+            }
+            if (ok || !SORTED) {                         // a sorted record fails only its check (checks builds)
+                out_u[3 * idx + c] = u;
+                if (GRAD) {
+                    out_grad[9 * idx + 3 * c + 0] = gx * dscale;
+                    out_grad[9 * idx + 3 * c + 1] = gy * dscale;
+                    out_grad[9 * idx + 3 * c + 2] = gz * dscale;
+                }
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -1367,7 +1448,7 @@ template <typename K> int set_smem(K kernel, size_t bytes) {
 
 template <int ORD, typename CT, typename AT, typename TR>
 int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, void* out_u, void* out_grad,
-               bool grad) {
+               bool grad, unsigned below) {
     const unsigned NB = g.NB;
     const size_t sm = tile_bytes<ORD, CT>();
     const AT dscale = (AT)((double)p->N / p->L);
@@ -1401,8 +1482,11 @@ int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, voi
                           ? kTmaOn : 0;
         }
         if (use_tma && (p->test_hooks & BSPLINE_TEST_SKIP_TMA_ISSUE)) use_tma = kTmaArmOnly;
-        // work items: at most one partial chunk per brick plus P / kChunk full ones
-        const long long items = (long long)NB + (w.P + kChunk - 1) / kChunk;
+        // work items: at most one partial chunk per staged brick plus P / kChunk full ones; with a split a
+        // staged brick holds at least `below` particles (2^18 particles on 512^3: 44160 -> 8320 CTAs, of
+        // which most find no item, 43 -> 8 us)
+        const long long bricks = below ? std::min<long long>(NB, w.P / below) : NB;
+        const long long items = bricks + (w.P + kChunk - 1) / kChunk;
         k<<<(unsigned)items, kGatherThreads, sm_aligned, p->stream>>>(
             reinterpret_cast<const CT*>(coeffs), p->N, g, w, (float*)out_u, grad ? (float*)out_grad : nullptr, dscale,
             tmap, use_tma, p->d_status);
@@ -1410,23 +1494,24 @@ int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, voi
     return BSPLINE_OK;
 }
 
-// The direct gather of the bricks below the plan's split (FP32 accumulation only).
+// The direct gather (FP32 accumulation only): with x, of all P particles at their positions; without, of the
+// sorted particles of the bricks below the plan's split.
 template <int ORD, typename CT, typename AT, typename TR>
-int run_gather_direct(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, void* out_u, void* out_grad,
-                      bool grad, unsigned below) {
+int run_gather_points(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, Ws<TR> w, unsigned NB,
+                      void* out_u, void* out_grad, bool grad) {
     if constexpr (sizeof(AT) == 8) {
         return BSPLINE_OK;
     } else {
-        if (below == 0) return BSPLINE_OK;
-        const unsigned NB = g.NB;
-        const float dscale = (float)((double)p->N / p->L);
-        auto k = grad ? gather_direct<ORD, CT, TR, true> : gather_direct<ORD, CT, TR, false>;
-        // the sparse range's length is known on the device only: enough threads for every particle
-        // up to a few waves, grid-striding beyond
-        const long long want = (w.P + 255) / 256;
-        const unsigned blocks = (unsigned)std::max(1LL, std::min(want, 32LL * p->sms));
-        k<<<blocks, 256, 0, p->stream>>>(reinterpret_cast<const CT*>(coeffs), p->N, NB, w, (float*)out_u,
-                                         grad ? (float*)out_grad : nullptr, dscale, p->d_status);
+        const double scale = (double)p->N / p->L;
+        auto k = x ? (grad ? gather_points<ORD, CT, TR, true, false> : gather_points<ORD, CT, TR, false, false>)
+                   : (grad ? gather_points<ORD, CT, TR, true, true> : gather_points<ORD, CT, TR, false, true>);
+        // the sparse range's length is known on the device only: a few waves, grid-striding beyond
+        constexpr int G = Points<ORD, CT>::G;
+        const long long want = (P + G - 1) / G;
+        const unsigned blocks = (unsigned)std::min(want, x ? 1LL << 30 : 32LL * p->sms);
+        k<<<blocks, Points<ORD, CT>::T, 0, p->stream>>>(reinterpret_cast<const CT*>(coeffs), p->N, x, P, scale, NB, w,
+                                                        (float*)out_u, grad ? (float*)out_grad : nullptr, (float)scale,
+                                                        p->d_status);
         return BSPLINE_OK;
     }
 }
@@ -1436,14 +1521,13 @@ int run_gather_direct(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid
 #define BS_GATHER_EXTERN(ORD, CT, AT, TR)                                                                 \
     extern template int gather_impl::run_gather<ORD, CT, AT, TR>(bspline_plan_s*, const void*,               \
                                                                   gather_impl::Ws<TR>, BrickGrid, void*,     \
-                                                                  void*, bool);                              \
-    extern template int gather_impl::run_gather_direct<ORD, CT, AT, TR>(                                     \
-        bspline_plan_s*, const void*, gather_impl::Ws<TR>, BrickGrid, void*, void*, bool, unsigned);
+                                                                  void*, bool, unsigned);                              \
+    extern template int gather_impl::run_gather_points<ORD, CT, AT, TR>(                                     \
+        bspline_plan_s*, const void*, const double*, int64_t, gather_impl::Ws<TR>, unsigned, void*, void*, bool);
 #define BS_GATHER_INSTANTIATE(ORD, CT, AT, TR)                                                          \
     template int gather_impl::run_gather<ORD, CT, AT, TR>(bspline_plan_s*, const void*, gather_impl::Ws<TR>, \
-                                                           BrickGrid, void*, void*, bool);                  \
-    template int gather_impl::run_gather_direct<ORD, CT, AT, TR>(bspline_plan_s*, const void*,               \
-                                                                  gather_impl::Ws<TR>, BrickGrid, void*,     \
-                                                                  void*, bool, unsigned);
+                                                           BrickGrid, void*, void*, bool, unsigned);        \
+    template int gather_impl::run_gather_points<ORD, CT, AT, TR>(                                            \
+        bspline_plan_s*, const void*, const double*, int64_t, gather_impl::Ws<TR>, unsigned, void*, void*, bool);
 
 }  // namespace bs
