@@ -206,7 +206,8 @@ template <int ORD> struct FxShape {
     static constexpr int XP = ORD <= 5 ? 2 : 4;         // x parts of a brick
     static constexpr int XW = BX / XP;                   // origins of one part in x
     static constexpr int EX = XW + ORD - 1, EY = S::EY, EZ = S::EZ;
-    static constexpr int E3 = EX * EY * EZ;              // nodes of one component
+    static constexpr int PZ = (EZ + 3) & ~3;             // words of a z-row: whole 16-byte pieces
+    static constexpr int E3 = EX * EY * PZ;              // words of one component
 };
 static_assert(FxShape<2>::BX % FxShape<2>::XP == 0 && FxShape<8>::BX % FxShape<8>::XP == 0, "x parts");
 constexpr int kFxThreads = 384;
@@ -276,13 +277,15 @@ __global__ void cotangent_bound_kernel(const float* __restrict__ g_u, const floa
     if ((threadIdx.x & 31) == 0 && m) atomicMax(bound, m);
 }
 
-// The contributions of one particle to its 3 n^3 nodes (factorised as in spread_kernel), each handed to add(node, v).
-template <int ORD, bool GRAD, typename Add>
+// The contributions of one particle to its 3 n^3 nodes (factorised as in spread_kernel), handed to
+// add2(node, v) for the nodes node, node + 1 of a z-row together (packed two-way FP32 arithmetic, the same
+// operations per node), and to add1(node, v) for the last node of an odd row.
+template <int ORD, bool GRAD, typename Add2, typename Add1>
 __device__ __forceinline__ void spread_particle(const float (&cu)[3], const float (&cg)[9], float dscale,
                                                 const float (&wx)[ORD], const float (&dwx)[ORD],
                                                 const float (&wy)[ORD], const float (&dwy)[ORD],
                                                 const float (&wz)[ORD], const float (&dwz)[ORD], int base,
-                                                int E3, int EY, int EZ, Add add) {
+                                                int E3, int EY, int PZ, Add2 add2, Add1 add1) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const float gu = cu[c];
@@ -300,9 +303,18 @@ __device__ __forceinline__ void spread_particle(const float (&cu)[3], const floa
             for (int jy = 0; jy < ORD; ++jy) {
                 const float p0 = GRAD ? fmaf(q1, dwy[jy], q0 * wy[jy]) : q0 * wy[jy];
                 const float p1 = q2 * wy[jy];
-                const int line = base + c * E3 + (jx * EY + jy) * EZ;
+                const int line = base + c * E3 + (jx * EY + jy) * PZ;
+                const float2 p02 = make_float2(p0, p0), p12 = make_float2(p1, p1);
 #pragma unroll
-                for (int jz = 0; jz < ORD; ++jz) add(line + jz, GRAD ? fmaf(p1, dwz[jz], p0 * wz[jz]) : p0 * wz[jz]);
+                for (int jz = 0; jz + 1 < ORD; jz += 2) {
+                    float2 v = __fmul2_rn(p02, make_float2(wz[jz], wz[jz + 1]));
+                    if (GRAD) v = __ffma2_rn(p12, make_float2(dwz[jz], dwz[jz + 1]), v);
+                    add2(line + jz, v);
+                }
+                if (ORD % 2) {
+                    constexpr int jz = ORD - 1;
+                    add1(line + jz, GRAD ? fmaf(p1, dwz[jz], p0 * wz[jz]) : p0 * wz[jz]);
+                }
             }
         }
     }
@@ -316,10 +328,10 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
                  long long* __restrict__ acc_g, const unsigned* __restrict__ bound, float dscale, float bound_factor,
                  unsigned long long* __restrict__ status) {
     using F = FxShape<ORD>;
-    constexpr int EX = F::EX, EY = F::EY, EZ = F::EZ, E3 = F::E3, BZ = F::BZ, XW = F::XW;
+    constexpr int EX = F::EX, EY = F::EY, PZ = F::PZ, E3 = F::E3, XW = F::XW;
     const unsigned NB = bg.NB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned* hi = reinterpret_cast<unsigned*>(smem_raw);     // [3][EX][EY][EZ], then lo the same
+    unsigned* hi = reinterpret_cast<unsigned*>(smem_raw);     // [3][EX][EY][PZ], then lo the same
     unsigned* lo = hi + 3 * E3;
     unsigned brick, beg, end;
     if (!item_range(w, NB, blockIdx.x / F::XP, &brick, &beg, &end)) return;
@@ -330,7 +342,7 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
     __shared__ unsigned short s_order[kChunk];
     __shared__ unsigned s_gmax;
     const unsigned n = end - beg;
-    for (int e = threadIdx.x; e < 6 * E3; e += kFxThreads) hi[e] = 0u;
+    for (int e = threadIdx.x; e < 6 * E3 / 4; e += kFxThreads) reinterpret_cast<uint4*>(hi)[e] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < 32) s_bucket[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_gmax = 0;
     __syncthreads();
@@ -353,7 +365,7 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
             const bool ok = ox >= 0 && ox < F::BX && oy >= 0 && oy < F::BY && oz >= 0 && oz < F::BZ && idx < w.P;
             if (part == 0) (void)BS_CHECK_OK(ok, status + kStatusBounds);
             if (ok && ox / XW == part) {
-                const unsigned r = (unsigned)(((ox - part * XW) * EY + oy) * EZ + oz) & 31u;
+                const unsigned r = (unsigned)(((ox - part * XW) * EY + oy) * PZ + oz) & 31u;
                 packed[k] = (atomicAdd(&s_bucket[r], 1u) << 5) | r;
                 if (!DET && cot) {
                     const float4* cp4 = cot + 4 * (size_t)(beg + i);
@@ -394,7 +406,7 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
     const FxScale sc = DET ? fx_det_scale(gmax, bound_factor, w.P) : fx_item_scale(gmax, bound_factor, np);
     const float s1 = ldexpf(1.f, sc.e1), s2 = ldexpf(1.f, sc.e2);
     const int xs = part * XW;
-    auto particle = [&](const Rec<TR>& rc, unsigned slot, auto add) {
+    auto particle = [&](const Rec<TR>& rc, unsigned slot, auto add2, auto add1) {
         const int ox = (int)(rc.cell >> (2 * kAnchorBits)) - x0 - xs;
         const int oy = (int)((rc.cell >> kAnchorBits) & 1023u) - y0;
         const int oz = (int)(rc.cell & 1023u) - z0;
@@ -408,31 +420,48 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
         bspline_weights<ORD, float>((float)rc.t[0], wx, dwx);
         bspline_weights<ORD, float>((float)rc.t[1], wy, dwy);
         bspline_weights<ORD, float>((float)rc.t[2], wz, dwz);
-        spread_particle<ORD, GRAD>(cu, cg, dscale, wx, dwx, wy, dwy, wz, dwz, (ox * EY + oy) * EZ + oz, E3, EY, EZ,
-                                   add);
+        spread_particle<ORD, GRAD>(cu, cg, dscale, wx, dwx, wy, dwy, wz, dwz, (ox * EY + oy) * PZ + oz, E3, EY, PZ,
+                                   add2, add1);
     };
     // a thread's next record is requested while its current particle is spread
-    auto loop = [&](auto add) {
+    auto loop = [&](auto add2, auto add1) {
         Rec<TR> rc_next;
         if (threadIdx.x < np) rc_next = w.s_rec[beg + s_order[threadIdx.x]];
         for (unsigned q = threadIdx.x; q < np; q += kFxThreads) {
             const Rec<TR> rc = rc_next;
             const unsigned slot = beg + s_order[q];
             if (q + kFxThreads < np) rc_next = w.s_rec[beg + s_order[q + kFxThreads]];
-            particle(rc, slot, add);
+            particle(rc, slot, add2, add1);
         }
     };
     if (sc.fixed) {
-        loop([&](int node, float v) {
-            const float h = fmaf(v, s1, kRintMagic);
-            const float r = fmaf(v, s1, -(h - kRintMagic));  // exact: v 2^e1 - hi
-            const float l = fmaf(r, s2, kRintMagic);
-            red_shared_u32(hi + node, __float_as_uint(h) - kRintMagicBits);
-            red_shared_u32(lo + node, __float_as_uint(l) - kRintMagicBits);
-        });
+        const float2 s1p = make_float2(s1, s1), s2p = make_float2(s2, s2);
+        const float2 magic = make_float2(kRintMagic, kRintMagic), minus = make_float2(-1.f, -1.f);
+        loop(
+            [&](int node, float2 v) {
+                const float2 h = __ffma2_rn(v, s1p, magic);
+                const float2 r = __ffma2_rn(v, s1p, __ffma2_rn(h, minus, magic));   // exact: v 2^e1 - hi
+                const float2 l = __ffma2_rn(r, s2p, magic);
+                red_shared_u32(hi + node, __float_as_uint(h.x) - kRintMagicBits);
+                red_shared_u32(hi + node + 1, __float_as_uint(h.y) - kRintMagicBits);
+                red_shared_u32(lo + node, __float_as_uint(l.x) - kRintMagicBits);
+                red_shared_u32(lo + node + 1, __float_as_uint(l.y) - kRintMagicBits);
+            },
+            [&](int node, float v) {
+                const float h = fmaf(v, s1, kRintMagic);
+                const float r = fmaf(v, s1, -(h - kRintMagic));
+                const float l = fmaf(r, s2, kRintMagic);
+                red_shared_u32(hi + node, __float_as_uint(h) - kRintMagicBits);
+                red_shared_u32(lo + node, __float_as_uint(l) - kRintMagicBits);
+            });
     } else {
         float* acc = reinterpret_cast<float*>(hi);
-        loop([&](int node, float v) { red_shared_f32(acc + node, v); });
+        loop(
+            [&](int node, float2 v) {
+                red_shared_f32(acc + node, v.x);
+                red_shared_f32(acc + node + 1, v.y);
+            },
+            [&](int node, float v) { red_shared_f32(acc + node, v); });
     }
     __syncthreads();
     auto dst_row = [&](int row, auto* base) {
@@ -444,33 +473,30 @@ spread_fx_kernel(int N, BrickGrid bg, Ws<TR> w, const float4* __restrict__ cot, 
         for (int e = threadIdx.x; e < 3 * E3; e += kFxThreads) {
             const long long f = ((long long)(int)hi[e] << sc.e2) + (int)lo[e];
             if (f != 0) {
-                const int row = e / EZ, iz = e - row * EZ;
+                const int row = e / PZ, iz = e - row * PZ;           // the padding holds zeros
                 atomicAdd(reinterpret_cast<unsigned long long*>(dst_row(row, acc_g) + wrap_index(z0 + iz, N)),
                           (unsigned long long)f);
             }
         }
         return;
     }
-    // into g_coef: per tile row the brick's BZ nodes as BZ/4 aligned 16-byte vector atomics (z0 and N are
-    // multiples of 4, so 4 consecutive z stay inside one period), then the EZ - BZ halo nodes one by one
+    // into g_coef: a tile row as PZ / 4 aligned 16-byte vector atomics (z0 and N are multiples of 4, so 4
+    // consecutive z stay inside one period; the padding adds zeros)
     const float inv1 = ldexpf(1.f, -sc.e1), inv12 = ldexpf(1.f, -(sc.e1 + sc.e2));
-    auto value = [&](int node) {
-        return sc.fixed ? fmaf((float)(int)hi[node], inv1, (float)(int)lo[node] * inv12) : __uint_as_float(hi[node]);
-    };
-    constexpr int U = BZ / 4 + (EZ - BZ);
+    auto value = [&](unsigned h, unsigned l) { return fmaf((float)(int)h, inv1, (float)(int)l * inv12); };
+    constexpr int U = PZ / 4;
     for (int e = threadIdx.x; e < 3 * EX * EY * U; e += kFxThreads) {
         const int row = e / U, k = e - row * U;
-        float* dst = dst_row(row, g_coef);
-        if (k < BZ / 4) {
-            const int nd = row * EZ + 4 * k;
-            const float4 v = make_float4(value(nd), value(nd + 1), value(nd + 2), value(nd + 3));
-            if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f)
-                atomicAdd(reinterpret_cast<float4*>(dst + wrap_index(z0 + 4 * k, N)), v);
+        const uint4 h = reinterpret_cast<const uint4*>(hi)[e];
+        float4 v;
+        if (sc.fixed) {
+            const uint4 l = reinterpret_cast<const uint4*>(lo)[e];
+            v = make_float4(value(h.x, l.x), value(h.y, l.y), value(h.z, l.z), value(h.w, l.w));
         } else {
-            const int iz = BZ + (k - BZ / 4);
-            const float v = value(row * EZ + iz);
-            if (v != 0.f) atomicAdd(dst + wrap_index(z0 + iz, N), v);
+            v = make_float4(__uint_as_float(h.x), __uint_as_float(h.y), __uint_as_float(h.z), __uint_as_float(h.w));
         }
+        if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f)
+            atomicAdd(reinterpret_cast<float4*>(dst_row(row, g_coef) + wrap_index(z0 + 4 * k, N)), v);
     }
 }
 
