@@ -1072,6 +1072,35 @@ __device__ __forceinline__ void store_g9(float* p, unsigned odd, const float (&g
             odd ? make_float2(g[2 * k + 1], g[2 * k + 2]) : make_float2(g[2 * k], g[2 * k + 1]);
 }
 
+// Bank order of an item's particles.  Particles are bucketed by bank (bucket[0..31]: their counts) and
+// ordered rank-major, bank-minor: particle (bank r, rank k within it) comes after all of smaller rank and
+// after those of its rank in smaller banks.  tab[k] (k < kRankTable): the banks holding more than k
+// particles as a mask, and the particles of smaller rank; the warps of the CTA fill it, then synchronise.
+// Deeper ranks (a clump within one bank) are counted bank by bank.  Counting every particle that way took
+// 160 instructions each: 5 % of the quintic gather's, 8 % of the cubic position gradient's.
+constexpr unsigned kRankTable = 128;
+__device__ __forceinline__ void fill_rank_table(const unsigned* bucket, uint2* tab) {
+    const unsigned lane = threadIdx.x & 31, b = bucket[lane];
+    const unsigned top = min(__reduce_max_sync(0xffffffffu, b), kRankTable);
+    for (unsigned k = threadIdx.x >> 5; k < top; k += blockDim.x >> 5) {
+        const unsigned mask = __ballot_sync(0xffffffffu, b > k), below = __reduce_add_sync(0xffffffffu, min(b, k));
+        if (lane == 0) tab[k] = make_uint2(mask, below);
+    }
+}
+__device__ __forceinline__ unsigned bank_position(const unsigned* bucket, const uint2* tab, unsigned r, unsigned k) {
+    if (k < kRankTable) {
+        const uint2 t = tab[k];
+        return t.y + (unsigned)__popc(t.x & ((1u << r) - 1u));
+    }
+    unsigned pos = 0;
+#pragma unroll 8
+    for (unsigned q = 0; q < 32; ++q) {
+        const unsigned bq = bucket[q];
+        pos += min(bq, k) + ((q < r && bq > k) ? 1u : 0u);
+    }
+    return pos;
+}
+
 // FP32 accumulation (FP32 or BF16 coefficients).  Each particle reads
 // 3 ORD^3 tile values from shared memory, and a warp load costs one cycle per
 // distinct address in the busiest of the 32 banks; random stencil origins
@@ -1102,6 +1131,7 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
     // would be a generic one)
     float* tile = reinterpret_cast<float*>(smem_raw + ((0u - smem_u32(smem_raw)) & 127u));
     __shared__ unsigned s_bucket[32];
+    __shared__ uint2 s_rank[kRankTable];
     __shared__ unsigned short s_order[kChunk];
     __shared__ __align__(8) unsigned long long s_mbar;
     const unsigned brick = w.item[item];
@@ -1159,18 +1189,13 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
             }
         }
         __syncthreads();
-        // job-sorted position: all particles of smaller rank, then the same rank in smaller buckets
+        fill_rank_table(s_bucket, s_rank);
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             const int i = threadIdx.x + k * kGatherThreads;
             if (i < n) {
-                const unsigned r = packed[k] & 31u, rk = packed[k] >> 5;
-                unsigned pos = 0;
-#pragma unroll 8
-                for (unsigned q = 0; q < 32; ++q) {
-                    const unsigned bq = s_bucket[q];
-                    pos += min(bq, rk) + ((q < r && bq > rk) ? 1u : 0u);
-                }
+                const unsigned pos = bank_position(s_bucket, s_rank, packed[k] & 31u, packed[k] >> 5);
                 if (BS_CHECK_OK(pos < (unsigned)n, status + kStatusBounds)) s_order[pos] = (unsigned short)i;
             }
         }
