@@ -17,6 +17,7 @@
 #include <new>
 #include <vector>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace bs {
@@ -175,6 +176,16 @@ int upload_twiddles(bspline_plan_s* p) {
         t[m] = make_double2(re, im);
         tf[m] = make_float2((float)re, (float)im);
     }
+    if (p->d_twf) {
+        std::vector<int4> f(N);
+        for (int m = 0; m < N; ++m) {
+            const fixed::Limbs re = fixed::limbs(std::llrint(std::ldexp(t[m].x, 60)));
+            const fixed::Limbs im = fixed::limbs(std::llrint(std::ldexp(t[m].y, 60)));
+            f[m] = make_int4(re.hi, re.lo, im.hi, im.lo);
+        }
+        const cudaError_t e = cudaMemcpy(p->d_twf, f.data(), sizeof(int4) * N, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return set_cuda_error(e);
+    }
     cudaError_t e = cudaMemcpy(p->d_tw64, t.data(), sizeof(double2) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw32, tf.data(), sizeof(float2) * N, cudaMemcpyHostToDevice);
     return set_cuda_error(e);
@@ -226,6 +237,7 @@ void free_plan(bspline_plan_s* p) {
     if (p->d_c32) cudaFree(p->d_c32);
     if (p->d_tw64) cudaFree(p->d_tw64);
     if (p->d_tw32) cudaFree(p->d_tw32);
+    if (p->d_twf) cudaFree(p->d_twf);
     if (p->d_status) cudaFree(p->d_status);
     p->work.release();
     p->pws.release();
@@ -295,6 +307,7 @@ int bspline_plan(bspline_plan_t* out, int N, int order, bspline_dtype dtype) {
     if (e == cudaSuccess) e = cudaMalloc(&p->d_c32, sizeof(float) * N);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tw64, sizeof(double2) * N);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tw32, sizeof(float2) * N);
+    if (e == cudaSuccess && dtype == BSPLINE_F64) e = cudaMalloc(&p->d_twf, sizeof(int4) * N);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_status, sizeof(unsigned long long) * kStatusWords);
     if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(unsigned long long) * kStatusWords);
     if (e != cudaSuccess) {

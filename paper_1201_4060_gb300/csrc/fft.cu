@@ -23,12 +23,20 @@
 // Global accesses are coalesced along contiguous lines.  Radix-8/4/2 Stockham stages, fully
 // unrolled per transform length; twiddles exp(+2 pi i m / N) from a table
 // computed on the host in FP64.
-#include "fft_core.cuh"
+#include "fft_fixed.cuh"
 
 namespace bs {
 namespace {
 
 using namespace fftc;
+
+// FP64 transforms of more than one stage run in fixed point (fft_fixed.cuh).
+template <typename R, int N> constexpr bool fixed_stages() { return sizeof(R) == 8 && N > 16; }
+
+// Threads of a tile: whole warps for FP64, whose lines are reduced by shuffles.
+template <typename R, int L, int NL> constexpr int threads_of() {
+    return sizeof(R) == 8 ? (threads_for<L, NL>() + 31) & ~31 : threads_for<L, NL>();
+}
 
 // ---------------------------------------------------------------- pass X
 // Lines along kx (input stride N*H complex); batch index b = ky*H + kz is
@@ -40,12 +48,12 @@ using namespace fftc;
 // zero; they are not read, and the columns (ky, kz) outside the band are not
 // transformed or stored (the ky/kz pass never reads them).
 template <typename R, int N, int NL>
-__global__ void __launch_bounds__(threads_for<N, NL>())
+__global__ void __launch_bounds__(threads_of<R, N, NL>())
 fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __restrict__ out,
                 const R* __restrict__ c, const typename Cx<R>::T* __restrict__ tw, int comp0,
-                const typename Cx<R>::T* const* __restrict__ in_fields, int band) {
+                const typename Cx<R>::T* const* __restrict__ in_fields, int band, const int4* __restrict__ twf) {
     using V = typename Cx<R>::T;
-    constexpr int T = threads_for<N, NL>();
+    constexpr int T = threads_of<R, N, NL>();
     static_assert(T % NL == 0, "each thread stays on one line");
     constexpr int H = N / 2 + 1, HP = row_pitch(N);
     constexpr long long NH = (long long)N * H;
@@ -75,7 +83,8 @@ fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __r
         for (int b = 0; b < valid; ++b) any = any || col_in_band(b);
         if (!any) return;
     }
-    for (int m = t; m < N; m += T) tws[m] = tw[m];
+    if constexpr (!fixed_stages<R, N>())
+        for (int m = t; m < N; m += T) tws[m] = tw[m];
     // this thread's line: batch index b0 + bl = ky H + kz; prefilter c(ky) c(kz) of the line
     const int bl = t % NL;
     const long long bb = b0 + bl;
@@ -94,6 +103,22 @@ fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __r
     auto st = [&](int q, int b, V v) {
         if (col) dst[(long long)q * N * HP] = v;
     };
+    if constexpr (fixed_stages<R, N>()) {
+        __shared__ unsigned red[T / 32 * NL];
+        __shared__ int tops[NL];
+        Fx* fs = reinterpret_cast<Fx*>(s);
+        int4* ftw = reinterpret_cast<int4*>(tws);
+        for (int m = t; m < N; m += T) ftw[m] = twf[m];
+        LineScale scale;
+        if (stage_first_fixed<N, NL, T, NL>(fs, red, tops, ld, &scale)) {
+            stages_mid<Fx, N, NL, T, NL, radix_for(N)>(fs, ftw, 1);
+            stage_last<Fx, N, NL, T, NL, false>(fs, ftw, 1, [&](int q, int b, Fx v) {
+                if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
+            });
+            return;
+        }
+        for (int m = t; m < N; m += T) tws[m] = tw[m];
+    }
     if constexpr (radix_for(N) == N) {
         stage_single<V, N, NL, T>(ld, st);
     } else {
@@ -226,7 +251,7 @@ template <typename R, int N, int NL> constexpr int z_rows() {
 // multiple of 16 bytes modulo 128).
 template <typename V, int N> constexpr int z_row_pitch() { return row_pitch(N) + 16 / (int)sizeof(V); }
 
-// The fused kernel runs threads_for<N, TL> threads (TL = tile_lines) on Y
+// The fused kernel runs threads_of<R, N, TL> threads (TL = tile_lines) on Y
 // items of NLY columns and Z items of z_rows<R, N, TL> rows.
 template <typename R, int N, int TL, int NLY>
 constexpr size_t yz_smem_elems() {
@@ -238,19 +263,20 @@ constexpr size_t yz_smem_elems() {
     return N + (y > z ? y : z);
 }
 
-// CTAs per SM the fused kernel is compiled for: 32 warps per SM (FP32), 24 (FP64).
+// CTAs per SM the fused kernel is compiled for: 32 warps per SM (FP32), 16 (FP64: 128 registers).
 template <typename R, int N, int NL> constexpr int yz_min_blocks() {
-    constexpr int W = sizeof(R) == 4 ? 1024 : 768;
-    return (W / threads_for<N, NL>()) < 1 ? 1 : (W / threads_for<N, NL>());
+    constexpr int W = sizeof(R) == 4 ? 1024 : 512;
+    return (W / threads_of<R, N, NL>()) < 1 ? 1 : (W / threads_of<R, N, NL>());
 }
 
 template <typename R, typename OutT, int N, int NL, int NLY>
-__global__ void __launch_bounds__(threads_for<N, NL>(), yz_min_blocks<R, N, NL>())
+__global__ void __launch_bounds__(threads_of<R, N, NL>(), yz_min_blocks<R, N, NL>())
 fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, typename Cx<R>::T* ring,
              const typename Cx<R>::T* __restrict__ tw, unsigned* ctr, unsigned* error, int lag, int ring_slots,
-             int drop_signals, long long plane0, long long planes, OutT* const* __restrict__ out_fields, int band) {
+             int drop_signals, long long plane0, long long planes, OutT* const* __restrict__ out_fields, int band,
+             const int4* __restrict__ twf) {
     using V = typename Cx<R>::T;
-    constexpr int T = threads_for<N, NL>();
+    constexpr int T = threads_of<R, N, NL>();
     constexpr int H = N / 2 + 1, HP = row_pitch(N);
     constexpr int M = N / 2;
     constexpr int NR = z_rows<R, N, NL>();              // Z rows per item: same thread count as a Y item
@@ -270,7 +296,25 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
     unsigned* done_y = ctr + 1;
     unsigned* done_z = ctr + 1 + planes;
     const int t = threadIdx.x;
-    for (int m = t; m < N; m += T) tws[m] = tw[m];
+    constexpr bool FIXED = fixed_stages<R, N>();
+    __shared__ unsigned red[FIXED ? T / 32 * (NLY > NR ? NLY : NR) : 1];
+    __shared__ int tops[FIXED ? (NLY > NR ? NLY : NR) : 1];
+    Fx* fbuf = reinterpret_cast<Fx*>(buf);
+    int4* ftw = reinterpret_cast<int4*>(tws);
+    auto load_twiddles = [&]() {                        // visible after the next barrier
+        if constexpr (FIXED) {
+            for (int m = t; m < N; m += T) ftw[m] = twf[m];
+        } else {
+            for (int m = t; m < N; m += T) tws[m] = tw[m];
+        }
+    };
+    // an FP64 tile with values outside the fixed form's range: the FP64 twiddles for its stages
+    auto fp64_twiddles = [&]() {
+        __syncthreads();
+        for (int m = t; m < N; m += T) tws[m] = tw[m];
+        __syncthreads();
+    };
+    load_twiddles();
     // thread 0 claims the following item while this one runs (its counter round trip overlaps the work);
     // a claimed item depends only on earlier items, so the smallest running item can always proceed
     unsigned claimed = (t == 0) ? atomicAdd(next, 1u) : 0u;
@@ -342,14 +386,34 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
             auto st = [&](int q, int b, V v) {
                 if (b < valid) dst[(long long)q * HP + b] = v;
             };
-            if constexpr (radix_for(N) == N) {
-                if (t == 0) prefetch_flag();
-                stage_single<V, N, NLY, T>(ld, st);
-            } else {
-                stage_first<V, N, NLY, T, QY>(buf, ld);
-                if (t == 0) prefetch_flag();
-                stages_mid<V, N, NLY, T, QY, radix_for(N)>(buf, tws, 1);
-                stage_last<V, N, NLY, T, QY, false>(buf, tws, 1, st);
+            bool done = false;
+            if constexpr (FIXED) {
+                LineScale scale;
+                done = stage_first_fixed<N, NLY, T, QY>(fbuf, red, tops, ld, &scale);
+                if (done) {
+                    if (t == 0) prefetch_flag();
+                    stages_mid<Fx, N, NLY, T, QY, radix_for(N)>(fbuf, ftw, 1);
+                    stage_last<Fx, N, NLY, T, QY, false>(fbuf, ftw, 1, [&](int q, int b, Fx v) {
+                        if (b < valid) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
+                    });
+                } else {
+                    fp64_twiddles();
+                }
+            }
+            if (!done) {
+                if constexpr (radix_for(N) == N) {
+                    if (t == 0) prefetch_flag();
+                    stage_single<V, N, NLY, T>(ld, st);
+                } else {
+                    stage_first<V, N, NLY, T, QY>(buf, ld);
+                    if (t == 0) prefetch_flag();
+                    stages_mid<V, N, NLY, T, QY, radix_for(N)>(buf, tws, 1);
+                    stage_last<V, N, NLY, T, QY, false>(buf, tws, 1, st);
+                }
+                if constexpr (FIXED) {
+                    __syncthreads();
+                    load_twiddles();
+                }
             }
             __syncthreads();
             if (t == 0 && !drop_signals) {
@@ -393,12 +457,63 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
             }
             OutT* dst = ob + (lpl * N + y0) * (long long)N;
             auto st = [&](int m, int b, V z) { store_pair<OutT, V>(dst + (long long)b * N + 2 * m, z); };
-            if constexpr (radix_for(M) == M) {
-                stage_single<V, M, NR, T>(ld, st);
-            } else {
-                stage_first<V, M, NR, T, QZ, true>(trans, ld);
-                stages_mid<V, M, NR, T, QZ, radix_for(M)>(trans, tws, 2);
-                stage_last<V, M, NR, T, QZ, true>(trans, tws, 2, st);
+            bool done = false;
+            if constexpr (FIXED) {
+                // scale of each row (z = E + i O: at most 1 + sqrt 2 times the norms of its two modes, each of
+                // which two z share), the row's modes in fixed point in place, then the stages
+                constexpr int NT = T / NR;              // threads of a row
+                static_assert(T % NR == 0, "whole rows");
+                const int zb = t % NR, kmax = band ? band : M;
+                V* row = raw + zb * RP;
+                LineScale scale;
+                done = line_scale<NR, T>(
+                    [&](auto f) {
+                        for (int k = t / NR; k <= kmax; k += NT) {
+                            const V a = row[k];
+                            f((unsigned)__double2hiint(a.x), (unsigned)__double2loint(a.x));
+                            f((unsigned)__double2hiint(a.y), (unsigned)__double2loint(a.y));
+                        }
+                    },
+                    5, red, tops, &scale);
+                if (done) {
+                    for (int k = t / NR; k <= kmax; k += NT) {
+                        const V a = row[k];
+                        reinterpret_cast<Fx*>(row)[k] = Fx{scale.in(a.x), scale.in(a.y)};
+                    }
+                    __syncthreads();
+                    auto ldf = [&](int k, int b) -> Fx {
+                        const Fx* fr = reinterpret_cast<const Fx*>(raw + b * RP);
+                        const Fx zero = {0, 0};
+                        const Fx a = (!band || k <= band) ? fr[k] : zero;
+                        const Fx c = (!band || M - k <= band) ? fr[M - k] : zero;
+                        if (k == 0) return {a.x + c.x, a.x - c.x};
+                        const Fx bb = {c.x, -c.y};
+                        const Fx E = cadd(a, bb);
+                        const Fx O = twiddled(csub(a, bb), ftw[k]);
+                        return {E.x - O.y, E.y + O.x};
+                    };
+                    stage_first<Fx, M, NR, T, QZ, true>(fbuf, ldf);
+                    stages_mid<Fx, M, NR, T, QZ, radix_for(M)>(fbuf, ftw, 2);
+                    stage_last<Fx, M, NR, T, QZ, true>(fbuf, ftw, 2, [&](int m, int b, Fx z) {
+                        const LineScale sb(tops[b]);
+                        st(m, b, make_double2(sb.out(z.x), sb.out(z.y)));
+                    });
+                } else {
+                    fp64_twiddles();
+                }
+            }
+            if (!done) {
+                if constexpr (radix_for(M) == M) {
+                    stage_single<V, M, NR, T>(ld, st);
+                } else {
+                    stage_first<V, M, NR, T, QZ, true>(trans, ld);
+                    stages_mid<V, M, NR, T, QZ, radix_for(M)>(trans, tws, 2);
+                    stage_last<V, M, NR, T, QZ, true>(trans, tws, 2, st);
+                }
+                if constexpr (FIXED) {
+                    __syncthreads();
+                    load_twiddles();
+                }
             }
             __syncthreads();                            // smem is reused by the next item
         }
@@ -428,7 +543,7 @@ template <typename R, typename OutT, int N>
 int run_fft(bspline_plan_s* p, const void* u_hat, void* coeffs, int c0, int c1) {
     using V = typename Cx<R>::T;
     constexpr int NL = tile_lines<R>();
-    constexpr int T = threads_for<N, NL>();
+    constexpr int T = threads_of<R, N, NL>();
     constexpr int H = N / 2 + 1, HP = row_pitch(N);
     const R* c = nullptr;
     const V* tw = nullptr;
@@ -450,8 +565,8 @@ int run_fft(bspline_plan_s* p, const void* u_hat, void* coeffs, int c0, int c1) 
         if ((rc = set_smem(k, sm))) return rc;
         const long long tiles = ((long long)N * H + NLX - 1) / NLX;
         StageTimer tm(p, BSPLINE_STAGE_FFT_X);
-        k<<<(unsigned)((c1 - c0) * tiles), threads_for<N, NLX>(), sm, st>>>(reinterpret_cast<const V*>(u_hat), w, c,
-                                                                             tw, c0, nullptr, p->band);
+        k<<<(unsigned)((c1 - c0) * tiles), threads_of<R, N, NLX>(), sm, st>>>(reinterpret_cast<const V*>(u_hat), w, c,
+                                                                             tw, c0, nullptr, p->band, p->d_twf);
     }
     {
         auto k = fft_yz_fused<R, OutT, N, NL, kYCols * NL>;
@@ -479,7 +594,7 @@ int run_fft(bspline_plan_s* p, const void* u_hat, void* coeffs, int c0, int c1) 
         k<<<(unsigned)grid, T, sm, st>>>(w, reinterpret_cast<OutT*>(coeffs), ring, tw, ctr,
                                          reinterpret_cast<unsigned*>(p->d_status + kStatusTransformTimeout), lag, ring_slots,
                                          (p->test_hooks & BSPLINE_TEST_DROP_TRANSFORM_SIGNALS) ? 1 : 0,
-                                         (long long)c0 * N, planes, nullptr, p->band);
+                                         (long long)c0 * N, planes, nullptr, p->band, p->d_twf);
     }
     return set_cuda_error(cudaGetLastError());
 }
@@ -498,7 +613,7 @@ int run_fft_fields(const bspline_plan_s* p, int F, const void* const* in_fields,
                    unsigned* error, cudaStream_t st) {
     using V = typename Cx<R>::T;
     constexpr int NL = tile_lines<R>();
-    constexpr int T = threads_for<N, NL>();
+    constexpr int T = threads_of<R, N, NL>();
     constexpr int H = N / 2 + 1, HP = row_pitch(N);
     const R* c = nullptr;
     const V* tw = nullptr;
@@ -517,8 +632,8 @@ int run_fft_fields(const bspline_plan_s* p, int F, const void* const* in_fields,
         const size_t sm = sizeof(V) * (N + (size_t)N * NLX);
         if ((rc = set_smem(k, sm))) return rc;
         const long long tiles = ((long long)N * H + NLX - 1) / NLX;
-        k<<<(unsigned)(3LL * F * tiles), threads_for<N, NLX>(), sm, st>>>(
-            nullptr, w, c, tw, 0, reinterpret_cast<const V* const*>(in_fields), p->band);
+        k<<<(unsigned)(3LL * F * tiles), threads_of<R, N, NLX>(), sm, st>>>(
+            nullptr, w, c, tw, 0, reinterpret_cast<const V* const*>(in_fields), p->band, p->d_twf);
     }
     {
         auto k = fft_yz_fused<R, OutT, N, NL, kYCols * NL>;
@@ -540,7 +655,7 @@ int run_fft_fields(const bspline_plan_s* p, int F, const void* const* in_fields,
         e = cudaMemsetAsync(ctr, 0, sizeof(unsigned) * (1 + 2 * planes), st);
         if (e != cudaSuccess) return set_cuda_error(e);
         k<<<(unsigned)grid, T, sm, st>>>(w, nullptr, ring, tw, ctr, error, lag, 2 * lag, 0, 0LL, planes,
-                                         reinterpret_cast<OutT* const*>(out_fields), p->band);
+                                         reinterpret_cast<OutT* const*>(out_fields), p->band, p->d_twf);
     }
     return set_cuda_error(cudaGetLastError());
 }

@@ -21,6 +21,12 @@ template <typename V> __device__ __forceinline__ V csub(V a, V b) { return mk<V>
 template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
     return mk<V>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// Products with the butterflies' constants and with a twiddle (overloaded for the fixed-point form).
+template <typename R> __device__ __forceinline__ R mul_sqrt_half(R v) { return v * (R)0.70710678118654752440084436210485; }
+template <typename R> __device__ __forceinline__ R mul_half_sqrt3(R v) { return v * (R)0.86602540378443864676372317075294; }
+template <typename R> __device__ __forceinline__ R sub_half(R a, R s) { return a - (R)0.5 * s; }
+__device__ __forceinline__ float2 twiddled(float2 a, float2 w) { return cmul(a, w); }
+__device__ __forceinline__ double2 twiddled(double2 a, double2 w) { return cmul(a, w); }
 template <typename V> __device__ __forceinline__ V cmuli(V a) { return mk<V>(-a.y, a.x); }  // a * (+i)
 
 // Inverse DFTs (exponent +2 pi i n k / R) in registers.
@@ -37,15 +43,13 @@ template <typename V> __device__ __forceinline__ void dft4(V& x0, V& x1, V& x2, 
     x3 = csub(t1, t3);
 }
 template <typename V> __device__ __forceinline__ void dft8(V* x) {
-    using R = decltype(V::x);
     V e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
     V o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
     dft4(e0, e1, e2, e3);
     dft4(o0, o1, o2, o3);
-    const R s = (R)0.70710678118654752440084436210485;
-    V w1 = mk<V>((o1.x - o1.y) * s, (o1.x + o1.y) * s);     // exp(i pi/4) o1
-    V w2 = cmuli(o2);                                        // exp(i pi/2) o2
-    V w3 = mk<V>((-o3.x - o3.y) * s, (o3.x - o3.y) * s);    // exp(3 i pi/4) o3
+    V w1 = mk<V>(mul_sqrt_half(o1.x - o1.y), mul_sqrt_half(o1.x + o1.y));     // exp(i pi/4) o1
+    V w2 = cmuli(o2);                                                          // exp(i pi/2) o2
+    V w3 = mk<V>(mul_sqrt_half(-o3.x - o3.y), mul_sqrt_half(o3.x - o3.y));    // exp(3 i pi/4) o3
     x[0] = cadd(e0, o0);
     x[4] = csub(e0, o0);
     x[1] = cadd(e1, w1);
@@ -58,11 +62,9 @@ template <typename V> __device__ __forceinline__ void dft8(V* x) {
 // Length 3: with w = exp(2 pi i / 3) = -1/2 + i sqrt(3)/2, X1 and X2 are
 // a - (b + c)/2 +- i (sqrt(3)/2) (b - c).
 template <typename V> __device__ __forceinline__ void dft3(V& a, V& b, V& c) {
-    using R = decltype(V::x);
-    const R h = (R)0.86602540378443864676372317075294;   // sqrt(3) / 2
     const V s = cadd(b, c), d = csub(b, c);
-    const V m = mk<V>(a.x - (R)0.5 * s.x, a.y - (R)0.5 * s.y);
-    const V id = mk<V>(-h * d.y, h * d.x);
+    const V m = mk<V>(sub_half(a.x, s.x), sub_half(a.y, s.y));
+    const V id = mk<V>(-mul_half_sqrt3(d.y), mul_half_sqrt3(d.x));
     a = cadd(a, s);
     b = cadd(m, id);
     c = csub(m, id);
@@ -79,8 +81,8 @@ template <int R, typename V> __device__ __forceinline__ void butterfly(V* v) {
 // Butterfly j of a line reads positions j + r L/R, multiplies by
 // exp(2 pi i r (j mod NS) / (NS R)), and writes positions
 // (j / NS) NS R + (j mod NS) + r NS.  All reads finish before any write.
-template <typename V, int L, int NLINES, int T, int RADIX, int NS, int QS>
-__device__ __forceinline__ void stage(V* s, const V* tw, int twstride) {
+template <typename V, int L, int NLINES, int T, int RADIX, int NS, int QS, typename W>
+__device__ __forceinline__ void stage(V* s, const W* tw, int twstride) {
     constexpr int NB = (L / RADIX) * NLINES;
     constexpr int BPT = (NB + T - 1) / T;
     V v[BPT][RADIX];
@@ -93,7 +95,7 @@ __device__ __forceinline__ void stage(V* s, const V* tw, int twstride) {
 #pragma unroll
             for (int r = 0; r < RADIX; ++r) {
                 V a = s[(j + r * (L / RADIX)) * QS + b];
-                if (NS > 1 && r > 0) a = cmul(a, tw[(r * k * (L / (NS * RADIX))) * twstride]);
+                if (NS > 1 && r > 0) a = twiddled(a, tw[(r * k * (L / (NS * RADIX))) * twstride]);
                 v[i][r] = a;
             }
             butterfly<RADIX>(v[i]);
@@ -176,8 +178,8 @@ __device__ __forceinline__ void stage_first(V* s, Ld ld) {
 }
 
 // Stages after the first, up to (not including) the last.
-template <typename V, int L, int NLINES, int T, int QS, int NS>
-__device__ __forceinline__ void stages_mid(V* s, const V* tw, int twstride) {
+template <typename V, int L, int NLINES, int T, int QS, int NS, typename W>
+__device__ __forceinline__ void stages_mid(V* s, const W* tw, int twstride) {
     if constexpr (NS < ns_last(L)) {
         constexpr int RADIX = radix_for(L / NS);
         stage<V, L, NLINES, T, RADIX, NS, QS>(s, tw, twstride);
@@ -189,8 +191,8 @@ __device__ __forceinline__ void stages_mid(V* s, const V* tw, int twstride) {
 // exp(2 pi i r j / L), and hands output position j + r NS of line b to st.
 // Consecutive threads take consecutive lines (JFAST = false) or consecutive
 // butterflies of one line (JFAST = true: stores along a line coalesce).
-template <typename V, int L, int NLINES, int T, int QS, bool JFAST, typename St>
-__device__ __forceinline__ void stage_last(const V* s, const V* tw, int twstride, St st) {
+template <typename V, int L, int NLINES, int T, int QS, bool JFAST, typename W, typename St>
+__device__ __forceinline__ void stage_last(const V* s, const W* tw, int twstride, St st) {
     constexpr int NS = ns_last(L);
     constexpr int RADIX = L / NS;
     constexpr int NB = NS * NLINES;
@@ -205,7 +207,7 @@ __device__ __forceinline__ void stage_last(const V* s, const V* tw, int twstride
 #pragma unroll
             for (int r = 0; r < RADIX; ++r) {
                 V a = s[(j + r * NS) * QS + b];
-                if (r > 0) a = cmul(a, tw[(r * j) * twstride]);
+                if (r > 0) a = twiddled(a, tw[(r * j) * twstride]);
                 v[r] = a;
             }
             butterfly<RADIX>(v);

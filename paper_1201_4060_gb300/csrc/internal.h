@@ -105,6 +105,7 @@ struct bspline_plan_s {
     float* d_c32 = nullptr;
     double2* d_tw64 = nullptr;
     float2* d_tw32 = nullptr;
+    int4* d_twf = nullptr;  // FP64 plans: the twiddles in fixed point (re.hi, re.lo, im.hi, im.lo; fixed.cuh)
 
     // Transform workspace: complex [3][N][N][N/2+1].
     bs::DeviceBuffer work;
