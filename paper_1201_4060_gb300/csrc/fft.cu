@@ -33,9 +33,11 @@ using namespace fftc;
 // FP64 transforms of more than one stage run in fixed point (fft_fixed.cuh).
 template <typename R, int N> constexpr bool fixed_stages() { return sizeof(R) == 8 && N > 16; }
 
-// Threads of a tile: whole warps for FP64, whose lines are reduced by shuffles.
+// Threads of a tile.  Fixed point: twice as many, one butterfly each, because its unrolled stages otherwise
+// outgrow the instruction cache (6 of 10 stall cycles in the ky/kz pass) and the registers; whole warps,
+// for the shuffles that reduce a line.
 template <typename R, int L, int NL> constexpr int threads_of() {
-    return sizeof(R) == 8 ? (threads_for<L, NL>() + 31) & ~31 : threads_for<L, NL>();
+    return fixed_stages<R, L>() ? (2 * threads_for<L, NL>() + 31) & ~31 : threads_for<L, NL>();
 }
 
 // ---------------------------------------------------------------- pass X
@@ -263,9 +265,9 @@ constexpr size_t yz_smem_elems() {
     return N + (y > z ? y : z);
 }
 
-// CTAs per SM the fused kernel is compiled for: 32 warps per SM (FP32), 16 (FP64: 128 registers).
+// CTAs per SM the fused kernel is compiled for: 32 warps per SM (FP32), 20 (FP64).
 template <typename R, int N, int NL> constexpr int yz_min_blocks() {
-    constexpr int W = sizeof(R) == 4 ? 1024 : 512;
+    constexpr int W = sizeof(R) == 4 ? 1024 : 640;
     return (W / threads_of<R, N, NL>()) < 1 ? 1 : (W / threads_of<R, N, NL>());
 }
 
