@@ -58,25 +58,25 @@ fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __r
     constexpr int T = threads_of<R, N, NL>();
     static_assert(T % NL == 0, "each thread stays on one line");
     constexpr int H = N / 2 + 1, HP = row_pitch(N);
-    constexpr long long NH = (long long)N * H;
-    constexpr long long TILES = (NH + NL - 1) / NL;
+    constexpr unsigned NH = (unsigned)N * H;            // at most 1024 * 513: indices stay in 32 bits
+    constexpr unsigned TILES = (NH + NL - 1) / NL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tws = reinterpret_cast<V*>(smem_raw);
     V* s = tws + N;
     const int t = threadIdx.x;
     unsigned bx = blockIdx.x;
     if (in_fields) {
-        constexpr unsigned per = 3u * (unsigned)TILES;
+        constexpr unsigned per = 3u * TILES;
         const unsigned f = bx / per;
         bx -= f * per;
         in = in_fields[f];
         out += (long long)f * 3 * N * N * HP;
     }
     const int comp = comp0 + (int)(bx / TILES);
-    const long long b0 = (bx % TILES) * NL;
-    const int valid = (int)std::min<long long>(NL, NH - b0);
+    const unsigned b0 = (bx % TILES) * NL;
+    const int valid = (int)std::min<unsigned>(NL, NH - b0);
     auto col_in_band = [&](int b) {                      // column b0 + b = ky H + kz inside the band
-        const long long bb = b0 + b;
+        const unsigned bb = b0 + (unsigned)b;
         const int ky = (int)(bb / H), kz = (int)(bb % H);
         return kz <= band && (ky <= band || ky >= N - band);
     };
@@ -89,15 +89,17 @@ fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __r
         for (int m = t; m < N; m += T) tws[m] = tw[m];
     // this thread's line: batch index b0 + bl = ky H + kz; prefilter c(ky) c(kz) of the line
     const int bl = t % NL;
-    const long long bb = b0 + bl;
+    const unsigned bb = b0 + (unsigned)bl;
     const int ky = (int)(bb / H), kz = (int)(bb % H);
     const R cyz = (bl < valid) ? c[ky] * c[kz] : R(0);
     const V* src = in + (long long)comp * N * NH + b0;
     V* dst = out + (long long)comp * N * N * HP + (long long)ky * HP + kz;
     // this thread's line (every thread stays on its column bl: the b below is always bl)
     const bool col = bl < valid && (!band || col_in_band(bl));
+    // rows q that are read as zero: gap0 <= q < gap0 + gap (all of them beyond the columns)
+    const unsigned gap0 = col ? (unsigned)band + 1 : 0u, gap = col ? (band ? (unsigned)(N - 2 * band - 1) : 0u) : ~0u;
     auto ld = [&](int q, int b) -> V {                   // prefilter c(kx) c(ky) c(kz) on load
-        if (!col || (band && q > band && q < N - band)) return mk<V>(R(0), R(0));
+        if ((unsigned)q - gap0 < gap) return mk<V>(R(0), R(0));
         const V a = src[(long long)q * NH + b];
         const R f = __ldg(&c[q]) * cyz;
         return mk<V>(a.x * f, a.y * f);
@@ -268,7 +270,8 @@ constexpr size_t yz_smem_elems() {
 // CTAs per SM the fused kernel is compiled for: 32 warps per SM (FP32), 20 (FP64).
 template <typename R, int N, int NL> constexpr int yz_min_blocks() {
     constexpr int W = sizeof(R) == 4 ? 1024 : 640;
-    return (W / threads_of<R, N, NL>()) < 1 ? 1 : (W / threads_of<R, N, NL>());
+    constexpr int T = (threads_of<R, N, NL>() + 31) & ~31;     // whole warps take registers
+    return W / T < 1 ? 1 : W / T;
 }
 
 template <typename R, typename OutT, int N, int NL, int NLY>
@@ -381,12 +384,16 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
             const int valid = std::min(NLY, H - kz0);
             const V* src = w + pl * N * HP + kz0;
             V* dst = slot + kz0;
+            // rows q that are read as zero: gap0 <= q < gap0 + gap (all of them beyond the columns; a thread's
+            // column is t % NLY throughout)
+            const bool col = t % NLY < valid;
+            const unsigned gap0 = col ? (unsigned)band + 1 : 0u;
+            const unsigned gap = col ? (band ? (unsigned)(N - 2 * band - 1) : 0u) : ~0u;
             auto ld = [&](int q, int b) -> V {
-                return (b < valid && (!band || q <= band || q >= N - band)) ? __ldcs(&src[(long long)q * HP + b])
-                                                                              : mk<V>(R(0), R(0));
+                return (unsigned)q - gap0 < gap ? mk<V>(R(0), R(0)) : __ldcs(&src[(long long)q * HP + b]);
             };
             auto st = [&](int q, int b, V v) {
-                if (b < valid) dst[(long long)q * HP + b] = v;
+                if (col) dst[(long long)q * HP + b] = v;
             };
             bool done = false;
             if constexpr (FIXED) {
@@ -396,7 +403,7 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                     if (t == 0) prefetch_flag();
                     stages_mid<Fx, N, NLY, T, QY, radix_for(N)>(fbuf, ftw, 1);
                     stage_last<Fx, N, NLY, T, QY, false>(fbuf, ftw, 1, [&](int q, int b, Fx v) {
-                        if (b < valid) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
+                        if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
                     });
                 } else {
                     fp64_twiddles();
@@ -428,9 +435,14 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
             unsigned char* dstb = reinterpret_cast<unsigned char*>(raw);
             // with a band only the row's first band + 1 modes are staged (the others are read as zero)
             const int nch = band ? std::min(CHUNKS, ((band + 1) * (int)sizeof(V) + 15) / 16) : CHUNKS;
-            for (int j = t; j < NR * nch; j += T) {
-                const int row = j / nch, k = j - row * nch;
-                cp_async16_l2(dstb + (size_t)row * RP * sizeof(V) + 16 * k, src + (size_t)row * HP * sizeof(V) + 16 * k);
+            // T / NR threads a row, or 8 where that is fewer (no division by the run-time count of pieces: it was
+            // a quarter of the kernel's instructions)
+            constexpr int TR = T / NR > 8 ? T / NR : 8;
+            for (int row = t / TR; row < NR; row += T / TR) {
+                unsigned char* to = dstb + (size_t)row * RP * sizeof(V);
+                const unsigned char* from = src + (size_t)row * HP * sizeof(V);
+#pragma unroll 4
+                for (int k = t % TR; k < nch; k += TR) cp_async16_l2(to + 16 * k, from + 16 * k);
             }
             cp_async_wait_all();
             __syncthreads();                            // the slot's rows are read: release it
@@ -438,11 +450,12 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                 signal_release(&done_z[lp]);
                 prefetch_flag();
             }
+            const int kmax = band ? band : M;
             auto ld = [&](int k, int b) -> V {          // even/odd split of the half spectrum
                 const V* row = raw + b * RP;
                 const V zero = mk<V>(R(0), R(0));       // modes beyond the band
-                const V a = (!band || k <= band) ? row[k] : zero;
-                const V c = (!band || M - k <= band) ? row[M - k] : zero;   // k = 0: X[0] and X[M]
+                const V a = k <= kmax ? row[k] : zero;
+                const V c = M - k <= kmax ? row[M - k] : zero;       // k = 0: X[0] and X[M]
                 if (k == 0) return mk<V>(a.x + c.x, a.x - c.x);
                 const V bb = mk<V>(c.x, -c.y);
                 const V E = cadd(a, bb);
@@ -465,7 +478,7 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                 // which two z share), the row's modes in fixed point in place, then the stages
                 constexpr int NT = T / NR;              // threads of a row
                 static_assert(T % NR == 0, "whole rows");
-                const int zb = t % NR, kmax = band ? band : M;
+                const int zb = t % NR;
                 V* row = raw + zb * RP;
                 LineScale scale;
                 done = line_scale<NR, T>(
@@ -486,8 +499,8 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                     auto ldf = [&](int k, int b) -> Fx {
                         const Fx* fr = reinterpret_cast<const Fx*>(raw + b * RP);
                         const Fx zero = {0, 0};
-                        const Fx a = (!band || k <= band) ? fr[k] : zero;
-                        const Fx c = (!band || M - k <= band) ? fr[M - k] : zero;
+                        const Fx a = k <= kmax ? fr[k] : zero;
+                        const Fx c = M - k <= kmax ? fr[M - k] : zero;
                         if (k == 0) return {a.x + c.x, a.x - c.x};
                         const Fx bb = {c.x, -c.y};
                         const Fx E = cadd(a, bb);
