@@ -179,25 +179,20 @@ constexpr long long kWaitLimit = 1LL << 22;
 
 // Item index -> (plane, index within the plane: < TPZ for Y items, else TPZ + Z index).
 template <int TPZ, int ZPP>
-__device__ __forceinline__ void item_to_plane(long long item, long long planes, int lag, long long* pl, int* r) {
-    constexpr int IPP = TPZ + ZPP;
-    const long long head = (long long)lag * TPZ;                   // steps 0..lag-1: Y items only
-    const long long body = head + (planes - lag) * IPP;            // steps lag..planes-1: Y then Z
+__device__ __forceinline__ void item_to_plane(unsigned item, unsigned planes, unsigned lag, unsigned* pl, int* r) {
+    constexpr unsigned IPP = TPZ + ZPP;
+    const unsigned head = lag * TPZ;                               // steps 0..lag-1: Y items only
+    const unsigned body = head + (planes - lag) * IPP;             // steps lag..planes-1: Y then Z
     if (item < head) {
         *pl = item / TPZ;
         *r = (int)(item % TPZ);
     } else if (item < body) {
-        const long long j = item - head, s = lag + j / IPP;
+        const unsigned j = item - head, s = lag + j / IPP;
         const int q = (int)(j % IPP);
-        if (q < TPZ) {
-            *pl = s;
-            *r = q;
-        } else {
-            *pl = s - lag;
-            *r = q;
-        }
+        *pl = q < TPZ ? s : s - lag;
+        *r = q;
     } else {                                                       // steps planes..planes+lag-1: Z only
-        const long long j = item - body;
+        const unsigned j = item - body;
         *pl = planes + j / ZPP - lag;
         *r = TPZ + (int)(j % ZPP);
     }
@@ -296,7 +291,7 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
     V* buf = tws + N;                                   // Y: [N][QY] tile of NLY columns
     V* raw = buf;                                       // Z: NR ring rows, pitch RP
     V* trans = buf;                                     // Z: [M][QZ] transform buffer over them (in place)
-    __shared__ unsigned s_item[2];
+    __shared__ uint4 s_item[2];                         // item, plane within the launch, index in it, ring slot
     unsigned* next = ctr;
     unsigned* done_y = ctr + 1;
     unsigned* done_z = ctr + 1 + planes;
@@ -325,17 +320,17 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
     unsigned claimed = (t == 0) ? atomicAdd(next, 1u) : 0u;
     const unsigned total = (unsigned)(planes * IPP);
     unsigned pre_item = 0xffffffffu, pre_val = 0;       // thread 0: relaxed read of the next item's flag
+    unsigned lp = 0;                                    // thread 0: the place of the item looked at last
+    int r = 0;
     // the flag an item waits for: a Z item its plane's Y items, a Y item its ring slot
     auto flag_of = [&](unsigned item, const unsigned** f, unsigned* target) {
-        long long lp;
-        int r;
-        item_to_plane<TPZ, ZPP>(item, planes, lag, &lp, &r);
+        item_to_plane<TPZ, ZPP>(item, (unsigned)planes, (unsigned)lag, &lp, &r);
         *f = nullptr;
         if (r >= TPZ) {
             *f = &done_y[lp];
             *target = (unsigned)TPZ;
-        } else if (lp >= ring_slots) {
-            *f = &done_z[lp - ring_slots];
+        } else if (lp >= (unsigned)ring_slots) {
+            *f = &done_z[lp - (unsigned)ring_slots];
             *target = (unsigned)ZPP;
         }
     };
@@ -363,16 +358,15 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                     else ok = spin_acquire(f, target, error) ? 1u : 0u;
                 }
             }
-            s_item[it & 1u] = ok ? item : 0xfffffffeu;
+            s_item[it & 1u] = make_uint4(ok ? item : 0xfffffffeu, lp, (unsigned)r, lp % (unsigned)ring_slots);
         }
         __syncthreads();
-        const unsigned item = s_item[it & 1u];
-        if (item >= total) return;
-        long long lp;                                   // plane within this launch; pl = plane0 + lp
-        int r;
-        item_to_plane<TPZ, ZPP>(item, planes, lag, &lp, &r);
+        const uint4 place = s_item[it & 1u];
+        if (place.x >= total) return;
+        const unsigned lp = place.y;                    // plane within this launch; pl = plane0 + lp
+        const int r = (int)place.z;
         const long long pl = plane0 + lp;
-        V* slot = ring + (lp % ring_slots) * (long long)N * HP;
+        V* slot = ring + place.w * (long long)N * HP;
         if (r < TPZ && band && r * NLY > band) {
             // ---- Y item beyond the band: its columns are zero, and the Z items never read them
             if (t == 0) prefetch_flag();
