@@ -211,7 +211,8 @@ __device__ __forceinline__ void q_scan(const FieldDesc& f, unsigned chunk_len) {
 }
 
 template <int ORD, int BYO, bool GRAD>
-__global__ void __launch_bounds__(gather_impl::kGatherThreads, 2) batch_queue_kernel(Queue q) {
+__global__ void __launch_bounds__(gather_impl::gather_threads<ORD, float, BYO>(), gather_impl::gather_ctas<ORD, float, BYO>())
+batch_queue_kernel(Queue q) {
     __shared__ int s_task[4];                            // phase (-1: skip, 4: done), field, index, spare
     const int F = q.F;
     const unsigned Tc = q.task_pre[F];                   // count tasks (and placement tasks)
@@ -287,10 +288,11 @@ int launch_batch_queue(const Queue& q, int sms, cudaStream_t stream) {
     const size_t sm = gather_impl::tile_bytes<ORD, float, BYO>() + 128;
     int rc = gather_impl::set_smem(k, sm);
     if (rc) return rc;
+    constexpr int T = gather_impl::gather_threads<ORD, float, BYO>();
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, gather_impl::kGatherThreads, sm);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, T, sm);
     if (e != cudaSuccess) return set_cuda_error(e);
-    k<<<(unsigned)(std::max(per_sm, 1) * sms), gather_impl::kGatherThreads, sm, stream>>>(q);
+    k<<<(unsigned)(std::max(per_sm, 1) * sms), T, sm, stream>>>(q);
     return set_cuda_error(cudaGetLastError());
 }
 

@@ -253,7 +253,6 @@ __device__ __forceinline__ void brick_origin(unsigned brick, const BrickGrid& g,
     *x0 = (int)(t / (unsigned)g.nby) * BX;
 }
 
-constexpr int kGatherThreads = 384;
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
@@ -1072,6 +1071,15 @@ __device__ __forceinline__ void store_g9(float* p, unsigned odd, const float (&g
             odd ? make_float2(g[2 * k + 1], g[2 * k + 2]) : make_float2(g[2 * k], g[2 * k + 1]);
 }
 
+// Threads of a gather CTA: 384, two CTAs on an SM; 256 and three where three tiles fit (FP32 up to order 4):
+// with the couple of hundred particles that a brick often holds, half of twelve warps would have no job, and
+// a third tile's copy is in flight.  Order 4, 256^3, 178 particles a brick: 155 -> 105 us (64-field batch 3.50 -> 3.28 ms).
+template <int ORD, typename CT, int BYO = 0> constexpr bool three_tiles() {
+    return 3 * ((sizeof(CT) == 2 ? Bf16Pair<ORD, BYO>::bytes : tile_bytes<ORD, CT, BYO>()) + 7 * 1024) <= 227 * 1024;
+}
+template <int ORD, typename CT, int BYO = 0> constexpr int gather_threads() { return three_tiles<ORD, CT, BYO>() ? 256 : 384; }
+template <int ORD, typename CT, int BYO = 0> constexpr int gather_ctas() { return three_tiles<ORD, CT, BYO>() ? 3 : 2; }
+
 // Bank order of an item's particles.  Particles are bucketed by bank (bucket[0..31]: their counts) and
 // ordered rank-major, bank-minor: particle (bank r, rank k within it) comes after all of smaller rank and
 // after those of its rank in smaller banks.  tab[k] (k < kRankTable): the banks holding more than k
@@ -1124,7 +1132,7 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
                                                 float* __restrict__ out_grad, float dscale, const CUtensorMap* tmap,
                                                 int use_tma, unsigned long long* __restrict__ status) {
     using S = Shape<CT, ORD, BYO>;
-    constexpr int NW = kGatherThreads / 32;
+    constexpr int T = gather_threads<ORD, CT, BYO>(), NW = T / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // the tile 128-byte aligned (TMA destinations; the launch adds 128 bytes of slack), offset from the
     // shared array itself so that its loads stay shared-memory loads (an address rebuilt from an integer
@@ -1174,11 +1182,11 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
         if (threadIdx.x < 32) s_bucket[threadIdx.x] = 0;
         __syncthreads();                                  // the tile copies stay in flight while bucketing
         // bucket (bank residue of the stencil origin) and rank within it, kept in registers
-        constexpr int KT = (kChunk + kGatherThreads - 1) / kGatherThreads;
+        constexpr int KT = (kChunk + T - 1) / T;
         unsigned packed[KT];
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
-            const int i = threadIdx.x + k * kGatherThreads;
+            const int i = threadIdx.x + k * T;
             if (i < n) {
                 const unsigned cp = w.s_rec[c0 + i].cell;
                 const int ox = (int)(cp >> (2 * kAnchorBits)) - x0;
@@ -1193,7 +1201,7 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
-            const int i = threadIdx.x + k * kGatherThreads;
+            const int i = threadIdx.x + k * T;
             if (i < n) {
                 const unsigned pos = bank_position(s_bucket, s_rank, packed[k] & 31u, packed[k] >> 5);
                 if (BS_CHECK_OK(pos < (unsigned)n, status + kStatusBounds)) s_order[pos] = (unsigned short)i;
@@ -1318,7 +1326,7 @@ __device__ __forceinline__ void gather_f32_item(unsigned item, unsigned chunk_le
 }
 
 template <int ORD, typename CT, typename TR, bool GRAD>
-__global__ void __launch_bounds__(kGatherThreads, 2)
+__global__ void __launch_bounds__(gather_threads<ORD, CT>(), gather_ctas<ORD, CT>())
 gather_f32(const CT* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, float* __restrict__ out_u,
            float* __restrict__ out_grad, float dscale, const __grid_constant__ CUtensorMap tmap, int use_tma,
            unsigned long long* __restrict__ status) {
@@ -1512,7 +1520,7 @@ int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, voi
         // which most find no item, 43 -> 8 us)
         const long long bricks = below ? std::min<long long>(NB, w.P / below) : NB;
         const long long items = bricks + (w.P + kChunk - 1) / kChunk;
-        k<<<(unsigned)items, kGatherThreads, sm_aligned, p->stream>>>(
+        k<<<(unsigned)items, gather_threads<ORD, CT>(), sm_aligned, p->stream>>>(
             reinterpret_cast<const CT*>(coeffs), p->N, g, w, (float*)out_u, grad ? (float*)out_grad : nullptr, dscale,
             tmap, use_tma, p->d_status);
     }
