@@ -92,7 +92,7 @@ int ensure_streams(bspline_batch_s* b, int k) {
 
 using batch_impl::FieldDesc;
 
-constexpr unsigned kQueuePartsPerTask = 8192;       // particles of one count / placement task
+constexpr unsigned kQueuePartsPerTask = 4096;       // particles of one count / placement task
 
 // Whether the fields can run through the persistent queue: FP32 plans of one
 // order, u and grad u for every field with particles.

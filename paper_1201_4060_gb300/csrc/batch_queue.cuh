@@ -105,58 +105,44 @@ __device__ __forceinline__ unsigned q_warp_inclusive(unsigned v, unsigned lane) 
 }
 
 // Count task: locate particles [p0, p1) of a field and count them per brick
-// (the single-field count pass, warp-aggregated increments).
+// (the single-field count pass); smem: `words` words of shared memory, used as
+// a histogram where it holds the field's bricks and the task's particles.
 template <int ORD>
-__device__ __forceinline__ void q_count(const FieldDesc& f, long long p0, long long p1, unsigned long long* status) {
-    const unsigned NB = f.bg.NB;
-    const int lane = threadIdx.x & 31;
-    for (long long pw = p0 + (threadIdx.x & ~31u); pw < p1; pw += blockDim.x) {
-        const long long p = pw + lane;
-        const bool valid = p < p1;
-        unsigned k = 0;
-        if (valid) {
-            Rec<float> r;
-            k = gather_impl::locate_particle<float>(f.x, p, f.N, f.scale, ORD, f.bg, &r);
-            if (k == NB) atomicAdd(&status[kStatusNonfinite], 1ULL);
-        }
-        const unsigned active = __ballot_sync(0xffffffffu, valid);
-        if (valid) {
-            const unsigned peers = __match_any_sync(active, k);
-            const unsigned leader = __ffs(peers) - 1;
-            if ((unsigned)lane == leader) atomicAdd(&f.w.count[k], (unsigned)__popc(peers));
-        }
+__device__ __forceinline__ void q_count(const FieldDesc& f, long long p0, long long p1, unsigned* smem, unsigned words,
+                                        unsigned long long* status) {
+    const unsigned NB = f.bg.NB, n = (unsigned)(p1 - p0);
+    auto key = [&](unsigned i) -> unsigned {
+        if (i >= n) return 0u;
+        Rec<float> r;
+        const unsigned k = gather_impl::locate_particle<float>(f.x, p0 + i, f.N, f.scale, ORD, f.bg, &r);
+        if (k == NB) atomicAdd(&status[kStatusNonfinite], 1ULL);
+        return k;
+    };
+    if (NB < (1u << gather_impl::kHistKeyBits) && NB + 1 + n <= words) {
+        gather_impl::count_run(smem, NB, n, f.w.count, f.w.rank + p0, key);
+    } else {
+        for (unsigned i = threadIdx.x; i < n; i += blockDim.x) f.w.rank[p0 + i] = atomicAdd(&f.w.count[key(i)], 1u);
     }
 }
 
-// Placement task: locate again and write each record to its brick's next slot; NaN outputs for
+// Placement task: locate again and write each record to its place in its brick's segment; NaN outputs for
 // non-finite positions.
 template <int ORD, bool GRAD>
 __device__ __forceinline__ void q_place(const FieldDesc& f, long long p0, long long p1,
                                         unsigned long long* status) {
     const unsigned NB = f.bg.NB;
-    const int lane = threadIdx.x & 31;
-    for (long long pw = p0 + (threadIdx.x & ~31u); pw < p1; pw += blockDim.x) {
-        const long long p = pw + lane;
+    for (long long p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
         Rec<float> r;
-        unsigned k = NB;
-        if (p < p1) k = gather_impl::locate_particle<float>(f.x, p, f.N, f.scale, ORD, f.bg, &r);
-        if (p < p1 && k >= NB) {
+        const unsigned k = gather_impl::locate_particle<float>(f.x, p, f.N, f.scale, ORD, f.bg, &r);
+        if (k >= NB) {
 #pragma unroll
             for (int i = 0; i < 3; ++i) f.out_u[3 * p + i] = NAN;
             if (GRAD) {
 #pragma unroll
                 for (int i = 0; i < 9; ++i) f.out_grad[9 * p + i] = NAN;
             }
-        }
-        const bool place = p < p1 && k < NB;
-        const unsigned active = __ballot_sync(0xffffffffu, place);
-        if (place) {
-            const unsigned peers = __match_any_sync(active, k);
-            const unsigned leader = __ffs(peers) - 1;
-            unsigned base = 0;
-            if ((unsigned)lane == leader) base = atomicAdd(&f.w.cursor[k], (unsigned)__popc(peers));
-            base = __shfl_sync(peers, base, leader);
-            const unsigned d = base + (unsigned)__popc(peers & ((1u << lane) - 1u));
+        } else {
+            const unsigned d = f.w.offset[k] + f.w.rank[p];
             r.idx = (unsigned)p;
             r.pad[0] = r.pad[1] = r.pad[2] = 0u;
             if (BS_CHECK_OK(d < f.w.offset[k] + f.w.count[k], status + kStatusBounds)) f.w.s_rec[d] = r;
@@ -164,7 +150,7 @@ __device__ __forceinline__ void q_place(const FieldDesc& f, long long p0, long l
     }
 }
 
-// Scan task: the field's brick offsets, cursors, item prefix and item -> brick
+// Scan task: the field's brick offsets, item prefix and item -> brick
 // map (every brick staged), by one CTA of any multiple of 32 threads.
 __device__ __forceinline__ void q_scan(const FieldDesc& f, unsigned chunk_len) {
     __shared__ unsigned wd[32], wc[32];
@@ -193,7 +179,6 @@ __device__ __forceinline__ void q_scan(const FieldDesc& f, unsigned chunk_len) {
         const unsigned exc = cc + (warp ? wc[warp - 1] : 0u) + vc - nc;
         if (i < NB) {
             w.offset[i] = exd;
-            w.cursor[i] = exd;
             w.chunk[i] = exc;
             for (unsigned k = 0; k < nc; ++k) w.item[exc + k] = i;
         }
@@ -203,7 +188,6 @@ __device__ __forceinline__ void q_scan(const FieldDesc& f, unsigned chunk_len) {
     }
     if (t == 0) {
         w.offset[NB] = cd;
-        w.cursor[NB] = cd;
         w.offset[NB + 1] = cd + w.count[NB];
         w.offset[NB + 2] = cd;
         w.chunk[NB] = cc;
@@ -213,6 +197,7 @@ __device__ __forceinline__ void q_scan(const FieldDesc& f, unsigned chunk_len) {
 template <int ORD, int BYO, bool GRAD>
 __global__ void __launch_bounds__(gather_impl::gather_threads<ORD, float, BYO>(), gather_impl::gather_ctas<ORD, float, BYO>())
 batch_queue_kernel(Queue q) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_task[4];                            // phase (-1: skip, 4: done), field, index, spare
     const int F = q.F;
     const unsigned Tc = q.task_pre[F];                   // count tasks (and placement tasks)
@@ -261,7 +246,9 @@ batch_queue_kernel(Queue q) {
         if (phase == 0 || phase == 2) {
             const long long p0 = (long long)j * q.part_per_task;
             const long long p1 = min(f.P, p0 + (long long)q.part_per_task);
-            if (phase == 0) q_count<ORD>(f, p0, p1, q.status);
+            if (phase == 0)
+                q_count<ORD>(f, p0, p1, reinterpret_cast<unsigned*>(smem_raw),
+                             (unsigned)(gather_impl::tile_bytes<ORD, float, BYO>() / sizeof(unsigned)), q.status);
             else q_place<ORD, GRAD>(f, p0, p1, q.status);
             __syncthreads();
             if (threadIdx.x == 0 && !(phase == 0 && q.drop_first_signal && fi == 0 && j == 0))

@@ -73,41 +73,31 @@ namespace {
 using namespace gather_impl;
 
 // ------------------------------------------------------------------ bin
-// Below this many bricks, particles of one warp often share a brick: aggregate their counter updates.
-constexpr unsigned kAggregateBricks = 4096;
-
 // Warp-aggregated increment of counter[key] for the lanes of `active`: one
-// atomic per distinct key in the warp (few bricks, many particles: small
-// grids); returns this lane's slot (old value + its rank among equal keys).
-__device__ __forceinline__ unsigned warp_increment(unsigned* counter, unsigned key, unsigned active, bool need_old) {
-    const unsigned lane = threadIdx.x & 31u;
+// atomic per distinct key in the warp (positions in brick order).
+__device__ __forceinline__ void warp_increment(unsigned* counter, unsigned key, unsigned active) {
     const unsigned peers = __match_any_sync(active, key);
-    const unsigned leader = __ffs(peers) - 1;
-    unsigned base = 0;
-    if (lane == leader) base = need_old ? atomicAdd(&counter[key], (unsigned)__popc(peers))
-                                        : (atomicAdd(&counter[key], (unsigned)__popc(peers)), 0u);
-    base = __shfl_sync(peers, base, leader);
-    return base + (unsigned)__popc(peers & ((1u << lane) - 1u));
+    if ((threadIdx.x & 31u) == __ffs(peers) - 1) atomicAdd(&counter[key], (unsigned)__popc(peers));
 }
 
 // Counting sort, pass 1: particles per brick (slot NB: invalid positions, also
-// counted in the status word).  The grid-stride loop runs warp-uniformly so that
-// lanes can aggregate their increments (aggregate = few bricks).  SORTED: the
+// counted in the status word).  HIST: runs of `run` particles, counted in shared
+// memory, which also gives each particle's place within its brick (count_run);
+// else one atomic a particle, and the placement pass draws the places.  Both
+// loops run warp-uniformly.  SORTED: the
 // caller passed the positions grouped by brick, so position p is also the
 // particle's sorted slot: its record is written there (coalesced, its own
 // index as the original one), each key is checked against its predecessor's
 // (the lane below, or located again at a warp's first lane) and *w.unsorted is
 // set if the order is broken anywhere, in which case the placement pass
 // rewrites every record; invalid positions get their NaN outputs here.
-template <typename TR, bool SORTED, typename OT>
-__global__ void bin_kernel(const double* __restrict__ x, long long P, int N, double scale, int order,
-                           BrickGrid g, Ws<TR> w, unsigned long long* __restrict__ status, int aggregate,
-                           OT* __restrict__ out_u, OT* __restrict__ out_grad) {
+template <typename TR, bool SORTED, bool HIST, typename OT>
+__global__ void __launch_bounds__(256)
+bin_kernel(const double* __restrict__ x, long long P, int N, double scale, int order, BrickGrid g, Ws<TR> w,
+           unsigned long long* __restrict__ status, unsigned run, OT* __restrict__ out_u, OT* __restrict__ out_grad) {
     const unsigned NB = g.NB;
-    const long long stride = (long long)gridDim.x * blockDim.x;
     const long long lane = threadIdx.x & 31;
-    for (long long pw = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; pw < P; pw += stride) {
-        const long long p = pw + lane;
+    auto key = [&](long long p) -> unsigned {            // every lane of the warp, consecutive p
         const bool valid = p < P;
         unsigned k = 0;
         if (valid) {
@@ -140,11 +130,25 @@ __global__ void bin_kernel(const double* __restrict__ x, long long P, int N, dou
                 }
             }
         }
-        if (aggregate) {
-            const unsigned active = __ballot_sync(0xffffffffu, valid);
-            if (valid) warp_increment(w.count, k, active, false);
-        } else if (valid) {
-            atomicAdd(&w.count[k], 1u);
+        return k;
+    };
+    if constexpr (HIST) {
+        extern __shared__ unsigned s_bin[];
+        for (long long p0 = (long long)blockIdx.x * run; p0 < P; p0 += (long long)gridDim.x * run)
+            count_run(s_bin, NB, (unsigned)min((long long)run, P - p0), w.count, w.rank + p0,
+                      [&](unsigned i) { return key(p0 + i); });
+    } else {
+        const long long stride = (long long)gridDim.x * blockDim.x;
+        for (long long pw = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; pw < P; pw += stride) {
+            const long long p = pw + lane;
+            const bool valid = p < P;
+            const unsigned k = key(p);
+            if constexpr (SORTED) {                      // a warp's particles share bricks
+                const unsigned active = __ballot_sync(0xffffffffu, valid);
+                if (valid) warp_increment(w.count, k, active);
+            } else if (valid) {
+                atomicAdd(&w.count[k], 1u);
+            }
         }
     }
 }
@@ -277,8 +281,8 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
 
 // ------------------------------------------------------------------ place
 // Counting sort, pass 2: locate again (cheaper than storing and re-reading the
-// records) and write each record and its original index to the next free slot
-// of its brick.  Invalid positions get NaN outputs.  SORTED: nothing to do
+// records) and write each record and its original index to its brick's segment:
+// at the place the count pass gave it (ranked), else at the next free slot.  Invalid positions get NaN outputs.  SORTED: nothing to do
 // unless the count pass found the order broken.  PERM (bspline_sort_order):
 // every particle, invalid ones included (bin NB, last), gets a slot, and only
 // its original index is written there, to perm.  cot (the adjoint of FP32
@@ -290,7 +294,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
 template <typename TR, typename OT, bool SORTED = false, bool PERM = false>
 __global__ void scatter_kernel(const double* __restrict__ x, long long P, int N, double scale, int order,
                                BrickGrid g, Ws<TR> w, OT* __restrict__ out_u, OT* __restrict__ out_grad,
-                               int aggregate, unsigned long long* __restrict__ status, int* __restrict__ perm = nullptr,
+                               int ranked, unsigned long long* __restrict__ status, int* __restrict__ perm = nullptr,
                                const float* __restrict__ cu = nullptr, const float* __restrict__ cg = nullptr,
                                float4* __restrict__ cot = nullptr) {
     const unsigned NB = g.NB;
@@ -302,7 +306,7 @@ __global__ void scatter_kernel(const double* __restrict__ x, long long P, int N,
         for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
             Rec<TR> r;
             const unsigned k = locate_particle<TR>(x, p, N, scale, order, g, &r);
-            const unsigned d = atomicAdd(&w.cursor[k], 1u);
+            const unsigned d = ranked ? w.offset[k] + w.rank[p] : atomicAdd(&w.cursor[k], 1u);
             if (BS_CHECK_OK(d < (unsigned)P, status + kStatusBounds)) perm[d] = (int)p;
         }
         return;
@@ -335,13 +339,7 @@ __global__ void scatter_kernel(const double* __restrict__ x, long long P, int N,
             for (int i = (int)lane; i < 9 * nq; i += 32) sw[96 + i] = cg ? cg[9 * pw + i] : 0.f;
             __syncwarp();
         }
-        unsigned d = 0;
-        if (aggregate) {
-            const unsigned active = __ballot_sync(0xffffffffu, place);
-            if (place) d = warp_increment(w.cursor, k, active, true);
-        } else if (place) {
-            d = atomicAdd(&w.cursor[k], 1u);
-        }
+        const unsigned d = !place ? 0u : (ranked ? w.offset[k] + w.rank[p] : atomicAdd(&w.cursor[k], 1u));
         if (place && BS_CHECK_OK(d < w.offset[k] + w.count[k], status + kStatusBounds)) {
             r.idx = (unsigned)p;
             if constexpr (sizeof(TR) == 4) r.pad[0] = r.pad[1] = r.pad[2] = 0u;
@@ -396,6 +394,32 @@ inline unsigned grid_for(long long P, int threads) {
     long long g = (P + threads - 1) / threads;
     if (g > (1LL << 30)) g = 1LL << 30;
     return (unsigned)(g < 1 ? 1 : g);
+}
+
+// The count pass; returns whether it ranked the particles.  Through shared-memory histograms where the bricks
+// are no more than a run's particles (the run, up to 8192, shrinks with P so that every SM gets two) or so few
+// that clustered particles queue for their counters: 2^22
+// particles, count + placement, 86 + 220 -> 63 + 223 us on 256^3 in the adjoint (5632 bricks, the cotangents'
+// copies bound the placement), 455 + 465 -> 55 + 76 us clustered on 128^3 (704 bricks, whose counters the
+// warps queued for).  Else an atomic a particle and pass: at 512^3 (44032 bricks, 2^24 particles) places
+// returned by the count's atomics made the step 1.5 % slower; at 5632 bricks and 10^6 particles the runs
+// (3328) gain nothing.
+template <typename TR, bool SORTED, typename OT>
+bool launch_bin(bspline_plan_s* p, const double* x, int64_t P, const BrickGrid& g, const Ws<TR>& w, OT* ou, OT* og,
+                unsigned grid, unsigned long long* status, cudaStream_t st) {
+    const double scale = (double)p->N / p->L;
+    const unsigned run = (unsigned)std::min<long long>(8192, std::max<long long>(1024, (P / (2 * p->sms) + 255) / 256 * 256));
+    if (g.NB <= std::max(run, 4096u)) {
+        const size_t sm = sizeof(unsigned) * (g.NB + 1 + run);
+        auto k = bin_kernel<TR, SORTED, true, OT>;
+        if (set_smem(k, sm) == BSPLINE_OK) {
+            const unsigned runs = (unsigned)((P + run - 1) / run);
+            k<<<std::min(runs, grid), 256, sm, st>>>(x, P, p->N, scale, p->order, g, w, status, run, ou, og);
+            return true;
+        }
+    }
+    bin_kernel<TR, SORTED, false, OT><<<grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, status, 0u, ou, og);
+    return false;
 }
 
 // Whether a call evaluates its particles in the caller's order, each straight from global memory
@@ -480,11 +504,11 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     unsigned below = p->direct_below;
     if (below == BSPLINE_GATHER_SPLIT_AUTO) below = auto_split(P, NB, p->order);
     if (sizeof(AT) == 8 || presorted) below = 0u;       // sorted input: bricks stay in input order
-    const int agg = NB < kAggregateBricks || presorted;  // sorted input: a warp's particles share bricks
+    bool ranked;
     {
         StageTimer tm(p, BSPLINE_STAGE_BIN);
-        if (presorted) bin_kernel<TR, true, AT><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, p->d_status, agg, ou, og);
-        else bin_kernel<TR, false, AT><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, p->d_status, agg, ou, og);
+        ranked = presorted ? launch_bin<TR, true, AT>(p, x, P, g, w, ou, og, sort_grid, p->d_status, st)
+                           : launch_bin<TR, false, AT>(p, x, P, g, w, ou, og, sort_grid, p->d_status, st);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
@@ -494,10 +518,10 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
         if (presorted)
-            scatter_kernel<TR, AT, true><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, ou, og, agg,
-                                                                    p->d_status);
+            scatter_kernel<TR, AT, true><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, ou, og,
+                                                                    ranked, p->d_status);
         else
-            scatter_kernel<TR, AT><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, ou, og, agg, p->d_status);
+            scatter_kernel<TR, AT><<<sort_grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, ou, og, ranked, p->d_status);
     }
     if (sort_stream) {
         if ((e = cudaEventRecord(sorted, sort_stream)) != cudaSuccess) return set_cuda_error(e);
@@ -534,11 +558,10 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     if ((e = cudaMemsetAsync(status, 0, sizeof(unsigned long long) * kStatusParticleWords, st)) != cudaSuccess)
         return set_cuda_error(e);                       // non-finite count, tile-wait flag, checks
     const bool grad = !(flags & BSPLINE_INTERP_NO_GRAD);
-    bin_kernel<TR, false, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, status,
-                                                               NB < kAggregateBricks, (AT*)nullptr, (AT*)nullptr);
+    const bool ranked = launch_bin<TR, false, AT>(p, x, P, g, w, nullptr, nullptr, grid_for(P, 256), status, st);
     scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len, P);
     scatter_kernel<TR, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, (AT*)out_u, grad ? (AT*)out_grad : nullptr,
-                                                             NB < kAggregateBricks, status);
+                                                             ranked, status);
     int rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, 0u);
     if (rc) return rc;
     return set_cuda_error(cudaGetLastError());
@@ -585,11 +608,10 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     if ((e = cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (NB + 2), st)) != cudaSuccess) return set_cuda_error(e);
     if ((e = cudaMemsetAsync(p->d_status, 0, sizeof(unsigned long long) * kStatusParticleWords, st)) != cudaSuccess)
         return set_cuda_error(e);                       // non-finite count, tile-wait flag, checks
+    bool ranked;
     {
         StageTimer tm(p, BSPLINE_STAGE_BIN);
-        bin_kernel<TR, false, double><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w,
-                                                                        p->d_status, NB < kAggregateBricks,
-                                                                        (double*)nullptr, (double*)nullptr);
+        ranked = launch_bin<TR, false, double>(p, x, P, g, w, nullptr, nullptr, grid_for(P, 256), p->d_status, st);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
@@ -598,7 +620,7 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
         const size_t cot_smem = cot ? sizeof(float) * 12 * 256 : 0;   // 12 * 32 floats per warp
-        scatter_kernel<TR, double><<<grid_for(P, 256), 256, cot_smem, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, g_x, nullptr, NB < kAggregateBricks,
+        scatter_kernel<TR, double><<<grid_for(P, 256), 256, cot_smem, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, g_x, nullptr, ranked,
                                                                      p->d_status, nullptr, (const float*)g_u,
                                                                      (const float*)g_grad, cot);
     }
@@ -637,13 +659,11 @@ int run_sort_order(bspline_plan_s* p, const double* x, int64_t P, int* perm) {
     if ((e = cudaMemsetAsync(p->d_status, 0, sizeof(unsigned long long) * kStatusParticleWords, st)) != cudaSuccess)
         return set_cuda_error(e);
     const double scale = (double)p->N / p->L;
-    const int agg = NB < kAggregateBricks;
-    bin_kernel<TR, false, float><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, p->d_status, agg,
-                                                                   (float*)nullptr, (float*)nullptr);
+    const bool ranked = launch_bin<TR, false, float>(p, x, P, g, w, nullptr, nullptr, grid_for(P, 256), p->d_status, st);
     scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk, P);
     scatter_kernel<TR, float, false, true><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w,
-                                                                            (float*)nullptr, (float*)nullptr, agg,
-                                                                            p->d_status, perm);
+                                                                            (float*)nullptr, (float*)nullptr,
+                                                                            ranked, p->d_status, perm);
     return set_cuda_error(cudaGetLastError());
 }
 

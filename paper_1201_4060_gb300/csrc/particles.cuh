@@ -55,7 +55,8 @@ template <typename TR> struct Ws {
     unsigned* unsorted; // nonzero if positions passed as sorted were not in brick order (count pass)
     unsigned* offset;   // [NB + 3]  start of each brick's sorted segment; [NB] end of the valid
                         //           particles, [NB + 1] end of all, [NB + 2] start of the sparse range
-    unsigned* cursor;   // [NB + 1]  next free sorted slot of each brick (starts at offset)
+    unsigned* cursor;   // [NB + 1]  next free sorted slot of each brick (starts at offset), without ranks
+    unsigned* rank;     // [P]       each particle's place within its brick (count pass by histograms)
     unsigned* chunk;    // [NB + 1]  exclusive prefix sum of ceil(count / chunk_len): first work item of a brick
     unsigned* item;     // [NB + ceil(P / chunk_len)]  brick of each work item (the first chunk[NB] are set)
     long long P;        // particles
@@ -76,6 +77,7 @@ template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t 
     w->unsorted = base ? w->count + NB + 1 : nullptr;
     w->offset = (unsigned*)take(sizeof(unsigned) * (NB + 3));
     w->cursor = (unsigned*)take(sizeof(unsigned) * (NB + 1));
+    w->rank = (unsigned*)take(sizeof(unsigned) * P);
     w->chunk = (unsigned*)take(sizeof(unsigned) * (NB + 1));
     w->item = (unsigned*)take(sizeof(unsigned) * (NB + (P + chunk_len - 1) / chunk_len));
     w->s_rec = (Rec<TR>*)take(sizeof(Rec<TR>) * P);
@@ -181,6 +183,35 @@ __device__ __forceinline__ unsigned locate_particle(const double* __restrict__ x
     r->t[1] = tt[1];
     r->t[2] = tt[2];
     return ((anc[0] >> g.bshift) * (unsigned)g.nby + anc[1] / (unsigned)g.by) * (unsigned)g.nbz + (anc[2] >> g.bshift);
+}
+
+// Count pass of a run of n particles by one CTA through a shared-memory histogram: key(i) gives the brick of
+// the run's i-th particle (each warp calls it for 32 consecutive i, all lanes; i >= n must return any key
+// and is not counted), count[] receives the run's counts, and rank[i] each particle's place within its
+// brick.  A global atomic per brick and run, on consecutive addresses, replaces one per particle and pass at
+// random ones: the placement pass then needs none.  s: NB + 1 + n words.
+constexpr unsigned kHistKeyBits = 14;                   // NB < 2^14, n <= 2^14
+template <typename Key>
+__device__ __forceinline__ void count_run(unsigned* s, unsigned NB, unsigned n, unsigned* __restrict__ count,
+                                          unsigned* __restrict__ rank, Key key) {
+    unsigned* s_key = s + NB + 1;
+    for (unsigned b = threadIdx.x; b <= NB; b += blockDim.x) s[b] = 0;
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < ((n + 31u) & ~31u); i += blockDim.x) {
+        const unsigned k = key(i);
+        if (i < n) s_key[i] = (atomicAdd(&s[k], 1u) << kHistKeyBits) | k;
+    }
+    __syncthreads();
+    for (unsigned b = threadIdx.x; b <= NB; b += blockDim.x) {
+        const unsigned h = s[b];
+        if (h) s[b] = atomicAdd(&count[b], h);
+    }
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+        const unsigned v = s_key[i];
+        rank[i] = s[v & ((1u << kHistKeyBits) - 1u)] + (v >> kHistKeyBits);
+    }
+    __syncthreads();
 }
 
 // ------------------------------------------------------------------ weights
