@@ -30,39 +30,59 @@ template <typename R, int N> constexpr int z_rows_adj() { return zr_rows<R>() < 
 // workspace [3][N][N][HP].  With T the inverse length-M transform of z and
 // Z[k] = T[(M - k) mod M] its forward transform:
 //   E[k] = (Z[k] + conj Z[M-k]) / 2,  O[k] = (Z[k] - conj Z[M-k]) / (2i),
-//   G[k] = E[k] + exp(-2 pi i k / N) O[k],  k = 0..M (indices mod M).
+//   G[k] = E[k] + exp(-2 pi i k / N) O[k],  G[M-k] = conj(E[k] - exp(-2 pi i k / N) O[k]),  k = 0..M/2
+// (indices mod M): a pair of modes from one pair of reads.  Bound: shared-memory passes.  The rows come in
+// 16-byte asynchronous copies and are transformed in place.
+template <typename V, int M> constexpr int zr_pitch() { return M + 16 / (int)sizeof(V); }   // rows skewed by 16 bytes
+template <typename R, int N> constexpr size_t zr_elems() {
+    constexpr size_t raw = (size_t)z_rows_adj<R, N>() * zr_pitch<typename Cx<R>::T, N / 2>();
+    constexpr size_t trans = (size_t)(N / 2) * (z_rows_adj<R, N>() + 1);
+    return raw > trans ? raw : trans;
+}
 template <typename R, int N>
 __global__ void __launch_bounds__(threads_for<N / 2, z_rows_adj<R, N>()>())
 fft_z_r2c(const R* __restrict__ g, typename Cx<R>::T* __restrict__ out, const typename Cx<R>::T* __restrict__ tw) {
     using V = typename Cx<R>::T;
-    constexpr int M = N / 2, NR = z_rows_adj<R, N>(), QZ = NR + 1;
+    constexpr int M = N / 2, NR = z_rows_adj<R, N>(), QZ = NR + 1, RP = zr_pitch<V, M>();
     constexpr int T = threads_for<M, NR>();
     constexpr int HP = row_pitch(N);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tws = reinterpret_cast<V*>(smem_raw);
-    V* trans = tws + N;
+    V* raw = tws + N;                                    // the rows as pairs of reals, then (in place)
+    V* trans = raw;                                      // the transform, [M][QZ]
     const int t = threadIdx.x;
     const long long r0 = (long long)blockIdx.x * NR;
-    for (int m = t; m < N; m += T) tws[m] = tw[m];
-    for (int e = t; e < NR * M; e += T) {
-        const int b = e / M, m = e % M;
-        const R* row = g + (r0 + b) * N;
-        trans[m * QZ + b] = mk<V>(row[2 * m], row[2 * m + 1]);
+    constexpr int CH = N * (int)sizeof(R) / 16;          // 16-byte pieces of a row
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(g + r0 * N);
+#pragma unroll 4
+    for (int e = t; e < NR * CH; e += T) {               // the rows are contiguous
+        const int b = e / CH, k = e % CH;
+        cp_async16(reinterpret_cast<unsigned char*>(raw + b * RP) + 16 * k, src + 16 * (size_t)e);
     }
+    for (int m = t; m < N; m += T) tws[m] = tw[m];
+    cp_async_wait_all();
     __syncthreads();
-    fft_smem<V, M, NR, T, QZ>(trans, tws, 2);
-    constexpr int H = M + 1;
-    for (int e = t; e < NR * H; e += T) {
-        const int b = e / H, k = e % H;
+    auto ld = [&](int k, int b) -> V { return raw[b * RP + k]; };
+    constexpr int NS = ns_last(M);
+    stage_first<V, M, NR, T, QZ, true>(trans, ld);
+    if constexpr (NS > 1) {
+        stages_mid<V, M, NR, T, QZ, radix_for(M)>(trans, tws, 2);
+        stage<V, M, NR, T, M / NS, NS, QZ>(trans, tws, 2);
+    }
+    constexpr int Q = M / 2 + 1;                         // pairs (k, M - k)
+    for (int e = t; e < NR * Q; e += T) {
+        const int b = e / Q, k = e % Q;
         const V zk = trans[((M - k) % M) * QZ + b];      // Z[k]
-        const V zm = trans[(k % M) * QZ + b];            // Z[M - k]
+        const V zm = trans[k * QZ + b];                  // Z[M - k]
         const V cm = mk<V>(zm.x, -zm.y);
         const V E = mk<V>((zk.x + cm.x) * R(0.5), (zk.y + cm.y) * R(0.5));
         const V d = csub(zk, cm);
         const V O = mk<V>(d.y * R(0.5), -d.x * R(0.5));   // d / (2i)
-        const V w = tws[k];                               // exp(+2 pi i k / N), k <= M < N
-        const V wc = mk<V>(w.x, -w.y);
-        out[(r0 + b) * HP + k] = cadd(E, cmul(wc, O));
+        const V w = tws[k];                               // exp(+2 pi i k / N)
+        const V wo = cmul(mk<V>(w.x, -w.y), O);
+        V* row = out + (r0 + b) * HP;
+        row[k] = cadd(E, wo);
+        if (2 * k != M) row[M - k] = mk<V>(E.x - wo.x, wo.y - E.y);
     }
 }
 
@@ -166,7 +186,7 @@ int run_adjoint_fft(bspline_plan_s* p, const void* g_coef, void* g_u_hat) {
         constexpr int NR = z_rows_adj<R, N>();
         constexpr int T = threads_for<N / 2, NR>();
         auto k = fft_z_r2c<R, N>;
-        const size_t sm = sizeof(V) * (N + (size_t)(N / 2) * (NR + 1));
+        const size_t sm = sizeof(V) * (N + zr_elems<R, N>());
         if ((rc = set_smem(k, sm))) return rc;
         k<<<(unsigned)(3LL * N * N / NR), T, sm, st>>>(reinterpret_cast<const R*>(g_coef), w, tw);
     }
