@@ -86,6 +86,20 @@ fft_z_r2c(const R* __restrict__ g, typename Cx<R>::T* __restrict__ out, const ty
     }
 }
 
+// The inverse transforms of a staged tile [N][NL], position q of line b handed to st(q, b, value): the first
+// stage in place, the last from shared memory to st.
+template <typename V, int N, int NL, int T, typename St>
+__device__ __forceinline__ void fft_staged(V* s, const V* tw, St st) {
+    auto ld = [&](int q, int b) -> V { return s[q * NL + b]; };
+    if constexpr (radix_for(N) == N) {
+        stage_single<V, N, NL, T>(ld, st);
+    } else {
+        stage_first<V, N, NL, T, NL, true>(s, ld);
+        stages_mid<V, N, NL, T, NL, radix_for(N)>(s, tw, 1);
+        stage_last<V, N, NL, T, NL, false>(s, tw, 1, st);
+    }
+}
+
 // ---------------------------------------------------------------- pass Y
 // One (component, x) plane, NL columns kz0.., all y: forward c2c along y in place.
 template <typename R, int N, int NL>
@@ -104,15 +118,13 @@ fft_y_fwd(typename Cx<R>::T* __restrict__ w, const typename Cx<R>::T* __restrict
     if (band && kz0 > band) return;                      // columns the band's last pass writes as zero
     const int valid = min(NL, H - kz0);
     V* base = w + pl * N * HP + kz0;
-    load_tile<V, N, NL, T, NL>(s, base, HP, valid);
+    load_tile<V, N, NL, T>(s, base, HP);                 // rows of HP: the columns beyond `valid` are padding
     for (int m = t; m < N; m += T) tws[m] = tw[m];
     cp_async_wait_all();
     __syncthreads();
-    fft_smem<V, N, NL, T, NL>(s, tws, 1);
-    for (int e = t; e < N * NL; e += T) {
-        const int q = e / NL, b = e % NL;
-        if (b < valid) base[(long long)q * HP + b] = s[((N - q) % N) * NL + b];
-    }
+    fft_staged<V, N, NL, T>(s, tws, [&](int q, int b, V v) {
+        if (b < valid) base[(long long)((N - q) % N) * HP + b] = v;
+    });
 }
 
 // ---------------------------------------------------------------- pass X
@@ -144,23 +156,20 @@ fft_x_fwd_prefilter(const typename Cx<R>::T* __restrict__ w, typename Cx<R>::T* 
         }
         return;
     }
-    load_tile<V, N, NL, T, NL>(s, w + (long long)comp * N * N * HP + (long long)ky * HP + kz0, (long long)N * HP,
-                               valid);
+    load_tile<V, N, NL, T>(s, w + (long long)comp * N * N * HP + (long long)ky * HP + kz0, (long long)N * HP);
     for (int m = t; m < N; m += T) tws[m] = tw[m];
     cp_async_wait_all();
     __syncthreads();
-    fft_smem<V, N, NL, T, NL>(s, tws, 1);
-    const R cy = __ldg(&c[ky]);
-    for (int e = t; e < N * NL; e += T) {
-        const int kx = e / NL, b = e % NL;
-        if (b < valid) {
-            const int kz = kz0 + b;
-            const R f = __ldg(&c[kx]) * cy * __ldg(&c[kz]) * ((kz == 0 || kz == M) ? R(1) : R(2));
-            const V a = s[((N - kx) % N) * NL + b];
-            const bool in = !band || (kz <= band && (kx <= band || kx >= N - band));
-            dst[((long long)kx * N + ky) * H + kz] = in ? mk<V>(a.x * f, a.y * f) : mk<V>(R(0), R(0));
-        }
-    }
+    static_assert(T % NL == 0, "a thread stays on its column");
+    const int kz = kz0 + t % NL;
+    const R cyz = t % NL < valid ? __ldg(&c[ky]) * __ldg(&c[kz]) * ((kz == 0 || kz == M) ? R(1) : R(2)) : R(0);
+    fft_staged<V, N, NL, T>(s, tws, [&](int q, int b, V a) {
+        if (b >= valid) return;
+        const int kx = (N - q) % N;
+        const R f = __ldg(&c[kx]) * cyz;
+        const bool in = !band || (kz <= band && (kx <= band || kx >= N - band));
+        dst[((long long)kx * N + ky) * H + kz] = in ? mk<V>(a.x * f, a.y * f) : mk<V>(R(0), R(0));
+    });
 }
 
 template <typename R, int N>

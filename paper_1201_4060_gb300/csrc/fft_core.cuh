@@ -121,20 +121,11 @@ constexpr int radix_for(int rem) {
     return (rem % 8 == 0) ? 8 : ((rem % 4 == 0) ? 4 : ((rem % 2 == 0) ? 2 : 3));
 }
 
-template <typename V, int L, int NLINES, int T, int QS, int NS = 1>
-__device__ __forceinline__ void fft_smem(V* s, const V* tw, int twstride) {
-    if constexpr (NS < L) {
-        constexpr int RADIX = radix_for(L / NS);
-        stage<V, L, NLINES, T, RADIX, NS, QS>(s, tw, twstride);
-        fft_smem<V, L, NLINES, T, QS, NS * RADIX>(s, tw, twstride);
-    }
-}
-
-// ---- the same transform with its first stage fed from registers and its
-// last stage written to registers, so the data make one trip through shared
-// memory fewer at each end (and the prefilter or pre/post-processing ride
+// ---- a transform has its first stage fed from registers and its last stage
+// written to registers, so the data make one trip through shared memory fewer
+// at each end (and the prefilter or pre/post-processing ride
 // along with the loads and stores).  The radix sequence is fixed by L:
-// radix_for(L / NS) at each stage, as in fft_smem.
+// radix_for(L / NS) at each stage.
 
 // NS of the last stage (NS * radix_for(L / NS) == L).
 constexpr int ns_last(int L) {
@@ -247,11 +238,6 @@ template <typename R> constexpr int tile_lines() { return sizeof(R) == 4 ? 8 : 4
 // H = N/2 + 1 rounded up to a multiple of 8, so every row starts 64-byte aligned.
 constexpr int row_pitch(int N) { return ((N / 2 + 1) + 7) & ~7; }
 
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                 "l"(src)
-                 : "memory");
-}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
                  "l"(src)
@@ -265,19 +251,16 @@ __device__ __forceinline__ void cp_async16_l2(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Copy a tile of NL-element row segments (row stride `pitch` elements) into
-// s[q * QS + b]; elements with b >= valid are zero.
-template <typename V, int ROWS, int NL, int T, int QS>
-__device__ __forceinline__ void load_tile(V* s, const V* __restrict__ src, long long pitch, int valid) {
-#pragma unroll
-    for (int e = threadIdx.x; e < ROWS * NL; e += T) {
-        const int q = e / NL, b = e % NL;
-        if (b < valid) {
-            if constexpr (sizeof(V) == 8) cp_async8(&s[q * QS + b], src + q * pitch + b);
-            else cp_async16(&s[q * QS + b], src + q * pitch + b);
-        } else {
-            s[q * QS + b] = mk<V>(0, 0);
-        }
+// Copy a tile of NL-element row segments (row stride `pitch` elements, segments and stride multiples of 16
+// bytes) into s[q * NL + b], in 16-byte pieces.
+template <typename V, int ROWS, int NL, int T>
+__device__ __forceinline__ void load_tile(V* s, const V* __restrict__ src, long long pitch) {
+    constexpr int E = 16 / (int)sizeof(V), P = NL / E;   // elements of a piece, pieces of a segment
+    static_assert(NL % E == 0, "whole pieces");
+#pragma unroll 4
+    for (int e = threadIdx.x; e < ROWS * P; e += T) {
+        const int q = e / P, k = e % P;
+        cp_async16(s + (size_t)q * NL + k * E, src + q * pitch + k * E);
     }
 }
 
