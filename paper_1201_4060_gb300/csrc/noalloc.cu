@@ -83,6 +83,7 @@ extern "C" int bspline_interp_noalloc(const void* coeffs, int N, int order, bspl
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return bs::set_cuda_error(e);
     p.device = dev;
+    if ((e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return bs::set_cuda_error(e);
     void* base = nullptr;
     int rc = scratch_for_device(dev, &base);
     if (rc == BSPLINE_OK) {
