@@ -514,7 +514,7 @@ static __global__ void det_finish_kernel(const long long* __restrict__ acc_g, fl
 
 // Position gradient: one thread per particle of the work item, coefficients
 // staged as in the forward evaluation.  FP32: bound by instruction issue and shared-memory latency; with
-// the y-lines in packed pairs and the ranked bank order 360 -> 327 us at 256^3 cubic, 2^22 particles.
+// the ranked bank order 360 -> 344 us at 256^3 cubic, 2^22 particles.
 template <int ORD, typename CT, typename TR, bool HESS>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(CT) == 8 ? 1 : 2)
 gx_kernel(const CT* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w,
@@ -622,46 +622,8 @@ gx_kernel(const CT* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w,
 #pragma unroll
             for (int jx = 0; jx < ORD; ++jx) {
                 A y00 = 0, y10 = 0, y01 = 0, y20 = 0, y02 = 0, y11 = 0;
-                int first = 0;
-                if constexpr (sizeof(A) == 4) {
-                    // y-lines in pairs, in packed two-way arithmetic (as the gather's row_x2)
-                    constexpr int NP = ORD / 2;
-                    float2 p00 = make_float2(0.f, 0.f), p10 = p00, p01 = p00, p20 = p00, p02 = p00, p11 = p00;
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        const float* l0 = reinterpret_cast<const float*>(tc) + jx * S::SX + 2 * p * S::SY;
-                        float2 z0v = make_float2(0.f, 0.f), z1v = z0v, z2v = z0v;
-#pragma unroll
-                        for (int jz = 0; jz < ORD; ++jz) {
-                            const float2 a = make_float2(l0[jz], l0[S::SY + jz]);
-                            z0v = __ffma2_rn(make_float2(wz[jz], wz[jz]), a, z0v);
-                            z1v = __ffma2_rn(make_float2(dwz[jz], dwz[jz]), a, z1v);
-                            if (HESS) z2v = __ffma2_rn(make_float2(d2wz[jz], d2wz[jz]), a, z2v);
-                        }
-                        const float2 w0 = make_float2(wy[2 * p], wy[2 * p + 1]);
-                        const float2 w1 = make_float2(dwy[2 * p], dwy[2 * p + 1]);
-                        p00 = __ffma2_rn(w0, z0v, p00);
-                        p10 = __ffma2_rn(w1, z0v, p10);
-                        p01 = __ffma2_rn(w0, z1v, p01);
-                        if (HESS) {
-                            p20 = __ffma2_rn(make_float2(d2wy[2 * p], d2wy[2 * p + 1]), z0v, p20);
-                            p02 = __ffma2_rn(w0, z2v, p02);
-                            p11 = __ffma2_rn(w1, z1v, p11);
-                        }
-                    }
-                    y00 = p00.x + p00.y;
-                    y10 = p10.x + p10.y;
-                    y01 = p01.x + p01.y;
-                    if (HESS) {
-                        y20 = p20.x + p20.y;
-                        y02 = p02.x + p02.y;
-                        y11 = p11.x + p11.y;
-                    }
-                    first = 2 * NP;
-                }
 #pragma unroll
                 for (int jy = 0; jy < ORD; ++jy) {
-                    if (jy < first) continue;            // FP64: every line; FP32: the last of an odd order
                     const A* line = tc + jx * S::SX + jy * S::SY;
                     A z0v = 0, z1v = 0, z2v = 0;
 #pragma unroll
