@@ -103,3 +103,36 @@ def test_non_finite_coefficients_reach_only_their_stencils(B, P):
     x = np.random.default_rng(6).uniform(0, L, (P, 3))
     u, _ = check(B, coef, x, N, order)
     assert 0 < np.isnan(u[:, 0]).sum() < P / 4 and np.isfinite(u[:, 1]).all()
+
+
+@pytest.mark.parametrize("N", [32, 48, 64])
+@pytest.mark.parametrize("scale", [1.0, 1e-250, 1e-300, 1e300])
+def test_transform_scales(B, N, scale):
+    """Spectra inside and outside the fixed-point range (2^-895 to 2^977), and tiles that mix both: one column
+    of modes 10^300 below its neighbours takes the FP64 stages with the rest of its tile."""
+    rng = np.random.default_rng(N)
+    half = rng.standard_normal((3, N, N, N // 2 + 1)) + 1j * rng.standard_normal((3, N, N, N // 2 + 1))
+    half[2] = 0.0
+    half *= scale
+    half[1, :, 1, 1] *= 1e-300
+    plan = B.Plan(N, 4, "f64")
+    c = plan.coeffs(torch.from_numpy(half).cuda()).cpu().numpy()
+    assert plan.status() == 0
+    ref = O.coefficients(half / scale, 4) * scale
+    assert (c[2] == 0).all()
+    for k in range(2):
+        assert np.abs(c[k] - ref[k]).max() <= 1e-12 * np.abs(ref[k]).max()
+    plan.close()
+
+
+def test_transform_non_finite_modes_reach_their_component(B):
+    N = 32
+    half = np.random.default_rng(1).standard_normal((3, N, N, N // 2 + 1)).astype(np.complex128)
+    ref = O.coefficients(half, 6)
+    half[0, 3, 4, 5] = np.nan
+    half[2, 0, 0, 0] = np.inf
+    plan = B.Plan(N, 6, "f64")
+    c = plan.coeffs(torch.from_numpy(half).cuda()).cpu().numpy()
+    assert np.isnan(c[0]).all() and not np.isfinite(c[2]).any()
+    assert np.abs(c[1] - ref[1]).max() <= 1e-12 * np.abs(ref[1]).max()
+    plan.close()
