@@ -146,8 +146,9 @@ int bspline_plan_set_stream(bspline_plan_t plan, void* stream);
  * with fewer than that many particles per brick on average and 0 otherwise;
  * bspline_plan_autotune picks the split by timing.  With AUTO and with "every
  * brick direct" (0xffffffff) a call of at most 12 Mi / n^3 particles (without
- * BSPLINE_INTERP_SORTED) is not sorted at all: the direct gather takes the
- * particles in the caller's order, without workspace. */
+ * BSPLINE_INTERP_SORTED; a quarter of that where the sort would run beside a
+ * transform, in bspline_eval and bspline_run_host) is not sorted at all: the
+ * direct gather takes the particles in the caller's order, without workspace. */
 #define BSPLINE_GATHER_SPLIT_AUTO 0xfffffffeu
 int bspline_plan_set_gather_split(bspline_plan_t plan, unsigned direct_below);
 

@@ -424,7 +424,7 @@ int bspline_eval(bspline_plan_t plan, const void* u_hat, void* coeffs, const dou
     if (!g.ok) return BSPLINE_ERR_CUDA;
     int rc;
     if (P == 0) return launch_coeffs(plan, u_hat, coeffs);
-    if (!interp_sorts(plan, P, flags)) {                // nothing to run beside the transform
+    if (!eval_sorts(plan, P, flags)) {                // nothing to run beside the transform
         if ((rc = launch_coeffs(plan, u_hat, coeffs))) return rc;
         return launch_interp(plan, coeffs, x, P, out_u, out_grad, flags);
     }
