@@ -127,25 +127,29 @@ BS_HD long long from_double(unsigned hi32, unsigned lo32, int emax) {
     return ((m ^ sign) - sign) >> (sh < 63 ? sh : 63);
 }
 
+BS_HD unsigned mul_hi(unsigned a, unsigned b) { return (unsigned)(((unsigned long long)a * b) >> 32); }
+
 // One component's sums over the stencil: the value and the three first derivatives in grid units, on the
 // values' scale.  at(jx, jy, jz) gives the limbs of a stencil value, wx(jx) the x weight of node jx and its
-// derivative weight (hi, lo, hi, lo).  *size: an upper estimate of the
-// largest |value|, the bitwise or of the magnitudes of the hi limbs.
+// derivative weight (hi, lo, hi, lo).  *size: a lower estimate of the weighted sum of magnitudes
+// sum w |a| that the results are rounded against, in units of 2^34: the y and x sums of |sum_z w a|, each
+// product rounded down.  It does not depend on GRAD.
 template <int n, bool GRAD, typename At, typename WX>
 BS_HD void contract(At at, WX wx, const Limbs (&wy)[n], const Limbs (&dwy)[n], const Limbs (&wz)[n],
-                    const Limbs (&dwz)[n], long long (&out)[4], int* size) {
+                    const Limbs (&dwz)[n], long long (&out)[4], unsigned* size) {
     Acc u, gx, gy, gz;
     u.clear();
     gx.clear();
     gy.clear();
     gz.clear();
-    int mag = 0;
+    unsigned sx = 0;
 #pragma unroll 1
     for (int jx = 0; jx < n; ++jx) {
         Acc y00, y10, y01;
         y00.clear();
         y10.clear();
         y01.clear();
+        unsigned sy = 0;
 #pragma unroll
         for (int jy = 0; jy < n; ++jy) {
             Acc z0, z1;
@@ -154,12 +158,12 @@ BS_HD void contract(At at, WX wx, const Limbs (&wy)[n], const Limbs (&dwy)[n], c
 #pragma unroll
             for (int jz = 0; jz < n; ++jz) {
                 const Limbs a = at(jx, jy, jz);
-                mag |= a.hi ^ (a.hi >> 31);
                 z0.add(a, wz[jz]);
                 if (GRAD) z1.add(a, dwz[jz]);
             }
             const Limbs l0 = z0.limbs();
             y00.add(l0, wy[jy]);
+            sy += mul_hi((unsigned)(l0.hi < 0 ? -l0.hi : l0.hi), (unsigned)wy[jy].hi);
             if (GRAD) {
                 y10.add(l0, dwy[jy]);
                 y01.add(z1.limbs(), wy[jy]);
@@ -169,6 +173,7 @@ BS_HD void contract(At at, WX wx, const Limbs (&wy)[n], const Limbs (&dwy)[n], c
         const int4 x = wx(jx);
         const Limbs w = {x.x, x.y};
         u.add(l00, w);
+        sx += mul_hi(sy, (unsigned)w.hi);
         if (GRAD) {
             gx.add(l00, {x.z, x.w});
             gy.add(y10.limbs(), w);
@@ -181,7 +186,7 @@ BS_HD void contract(At at, WX wx, const Limbs (&wy)[n], const Limbs (&dwy)[n], c
         out[2] = gy.value();
         out[3] = gz.value();
     }
-    *size = mag;
+    *size = sx;
 }
 
 }  // namespace fixed

@@ -860,15 +860,56 @@ __device__ __forceinline__ void eval_bf16(const unsigned* __restrict__ base, int
 }
 
 // u and grad u of one component of one particle in FP64 arithmetic, its stencil read from global memory
-// (comp: the component's [N][N][N] coefficients; a: the first stencil node).  The evaluation of the few
-// particles whose stencil the fixed-point form below does not represent: never inlined, rolled loops.
+// (comp: the component's [N][N][N] coefficients), for the particles whose stencil the fixed-point form below does
+// not hold: by one thread, or by a warp, with the same operations in the same order.  An FP64 instruction takes an
+// SM's quarter 75 cycles whatever its active lanes, so that one particle by one thread takes 15 (order 4) to 60 us
+// (order 8), as long as a small call's whole gather; a warp spreads the weights and the stencil's lines over its lanes.
+
+// One value of the recurrence of bspline_weights: M_k(t + m) from a = M_{k-1}(t + m), b = M_{k-1}(t + m - 1).
+template <int k> __device__ __forceinline__ double weight_f64(double t, int m, double a, double b) {
+    return fma(t + m, a, ((k - m) - t) * b) * (1.0 / (k - 1));
+}
+template <int n, int k = 2> __device__ __forceinline__ void weights_f64(double t, double (&v)[n], double (&w)[n], double (&dw)[n]) {
+    if constexpr (k == 2) {
+        v[0] = 1.0;
+#pragma unroll
+        for (int m = 1; m < n; ++m) v[m] = 0.0;
+    }
+    if constexpr (k < n) {
+#pragma unroll
+        for (int m = k - 1; m >= 0; --m) v[m] = weight_f64<k>(t, m, v[m], m > 0 ? v[m - 1] : 0.0);
+        weights_f64<n, k + 1>(t, v, w, dw);
+    } else {
+#pragma unroll
+        for (int m = 0; m < n; ++m) {
+            const double b = m > 0 ? v[m - 1] : 0.0;
+            w[n - 1 - m] = weight_f64<n>(t, m, v[m], b);
+            dw[n - 1 - m] = v[m] - b;
+        }
+    }
+}
+template <bool GRAD>
+__device__ __forceinline__ void store_f64(double u, double gx, double gy, double gz, double dscale,
+                                          double* __restrict__ out_u, double* __restrict__ out_grad) {
+    *out_u = u;
+    if (GRAD) {
+        out_grad[0] = gx * dscale;
+        out_grad[1] = gy * dscale;
+        out_grad[2] = gz * dscale;
+    }
+}
 template <int ORD, bool GRAD>
-__device__ __noinline__ void eval_f64_global(const double* __restrict__ comp, int N, int ax, int ay, int az, double tx,
-                                             double ty, double tz, double dscale, double* out) {
+__device__ __noinline__ void eval_f64_thread(const double* __restrict__ comp, int N, unsigned cell, double tx,
+                                             double ty, double tz, double dscale, double* __restrict__ out_u,
+                                             double* __restrict__ out_grad) {
+    const int ax = (int)(cell >> (2 * kAnchorBits)), ay = (int)((cell >> kAnchorBits) & 1023u), az = (int)(cell & 1023u);
     double wx[ORD], dwx[ORD], wy[ORD], dwy[ORD], wz[ORD], dwz[ORD];
-    bspline_weights<ORD, double>(tx, wx, dwx);
-    bspline_weights<ORD, double>(ty, wy, dwy);
-    bspline_weights<ORD, double>(tz, wz, dwz);
+    {
+        double v[ORD];
+        weights_f64<ORD>(tx, v, wx, dwx);
+        weights_f64<ORD>(ty, v, wy, dwy);
+        weights_f64<ORD>(tz, v, wz, dwz);
+    }
     double u = 0, gx = 0, gy = 0, gz = 0;
 #pragma unroll 1
     for (int jx = 0; jx < ORD; ++jx) {
@@ -877,7 +918,7 @@ __device__ __noinline__ void eval_f64_global(const double* __restrict__ comp, in
         for (int jy = 0; jy < ORD; ++jy) {
             const double* line = comp + ((size_t)wrap_index(ax + jx, N) * N + wrap_index(ay + jy, N)) * N;
             double z0 = 0, z1 = 0;
-#pragma unroll 1
+#pragma unroll
             for (int jz = 0; jz < ORD; ++jz) {
                 const double v = line[wrap_index(az + jz, N)];
                 z0 = fma(wz[jz], v, z0);
@@ -896,12 +937,84 @@ __device__ __noinline__ void eval_f64_global(const double* __restrict__ comp, in
             gz = fma(wx[jx], y01, gz);
         }
     }
-    out[0] = u;
-    if (GRAD) {
-        out[1] = gx * dscale;
-        out[2] = gy * dscale;
-        out[3] = gz * dscale;
+    store_f64<GRAD>(u, gx, gy, gz, dscale, out_u, out_grad);
+}
+
+// The recurrence with lane (axis, m) holding v[m]: after step k < n, M_k(t + m); then the node's two weights.
+template <int n, int k = 2> __device__ __forceinline__ void weights_f64_warp(double t, int m, double v, double* w, double* dw) {
+    double b = __shfl_up_sync(0xffffffffu, v, 1);
+    if (m == 0) b = 0.0;
+    if constexpr (k < n) {
+        weights_f64_warp<n, k + 1>(t, m, m < k ? weight_f64<k>(t, m, v, b) : 0.0, w, dw);
+    } else {
+        *w = weight_f64<n>(t, m, v, b);
+        *dw = v - b;
     }
+}
+template <int ORD, bool GRAD>
+__device__ __noinline__ void eval_f64_warp(const double* __restrict__ comp, int N, unsigned cell, double tx,
+                                           double ty, double tz, double dscale, double* __restrict__ out_u,
+                                           double* __restrict__ out_grad) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int R = (ORD * ORD + 31) / 32;             // lines of a lane
+    const int lane = threadIdx.x & 31;
+    const int ax = (int)(cell >> (2 * kAnchorBits)), ay = (int)((cell >> kAnchorBits) & 1023u), az = (int)(cell & 1023u);
+    double v[R][ORD];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int l = min(lane + 32 * r, ORD * ORD - 1), jx = l / ORD, jy = l % ORD;
+        const double* line = comp + ((size_t)wrap_index(ax + jx, N) * N + wrap_index(ay + jy, N)) * N;
+#pragma unroll
+        for (int jz = 0; jz < ORD; ++jz) v[r][jz] = line[wrap_index(az + jz, N)];
+    }
+    double w, dw;                                        // lane a ORD + m: node ORD - 1 - m of axis a
+    const int a = lane / ORD;
+    weights_f64_warp<ORD>(a == 0 ? tx : (a == 1 ? ty : tz), lane % ORD, lane % ORD == 0 ? 1.0 : 0.0, &w, &dw);
+    double z0[R], z1[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) z0[r] = z1[r] = 0.0;
+#pragma unroll
+    for (int jz = 0; jz < ORD; ++jz) {
+        const double wj = __shfl_sync(kAll, w, 3 * ORD - 1 - jz), dj = __shfl_sync(kAll, dw, 3 * ORD - 1 - jz);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            z0[r] = fma(wj, v[r][jz], z0[r]);
+            if (GRAD) z1[r] = fma(dj, v[r][jz], z1[r]);
+        }
+    }
+    double y00 = 0, y10 = 0, y01 = 0;                    // lane jx: the x-row's
+#pragma unroll
+    for (int jy = 0; jy < ORD; ++jy) {
+        const int l = min(lane, ORD - 1) * ORD + jy;
+        double a0 = 0, a1 = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double b0 = __shfl_sync(kAll, z0[r], l & 31), b1 = __shfl_sync(kAll, z1[r], l & 31);
+            if ((l >> 5) == r) {
+                a0 = b0;
+                a1 = b1;
+            }
+        }
+        const double wj = __shfl_sync(kAll, w, 2 * ORD - 1 - jy), dj = __shfl_sync(kAll, dw, 2 * ORD - 1 - jy);
+        y00 = fma(wj, a0, y00);
+        if (GRAD) {
+            y10 = fma(dj, a0, y10);
+            y01 = fma(wj, a1, y01);
+        }
+    }
+    double u = 0, gx = 0, gy = 0, gz = 0;
+#pragma unroll
+    for (int jx = 0; jx < ORD; ++jx) {
+        const double wj = __shfl_sync(kAll, w, ORD - 1 - jx), dj = __shfl_sync(kAll, dw, ORD - 1 - jx);
+        const double b00 = __shfl_sync(kAll, y00, jx);
+        u = fma(wj, b00, u);
+        if (GRAD) {
+            gx = fma(dj, b00, gx);
+            gy = fma(wj, __shfl_sync(kAll, y10, jx), gy);
+            gz = fma(wj, __shfl_sync(kAll, y01, jx), gz);
+        }
+    }
+    if (lane == 0) store_f64<GRAD>(u, gx, gy, gz, dscale, out_u, out_grad);
 }
 
 // FP64 plans: one CTA per work item, the brick's coefficients staged and turned into 60-bit fixed point
@@ -909,17 +1022,20 @@ __device__ __noinline__ void eval_f64_global(const double* __restrict__ comp, in
 // derivatives are integer multiply-adds, and only the twelve results are FP64 again.  Bound: integer issue.
 // The FP64 pipe took 1900 operations a particle at order 6: 5.36 ms for 10^6 particles on 256^3; the fixed
 // form's 5100 wide multiply-adds, with the tile's conversion (216 values a particle there), take 1.72 ms.
-// A stencil value is rounded at 2^-60 of the tile's largest, so the result is
-// at least as accurate as FP64 arithmetic (2^-53) for a stencil whose own largest value is within 2^kSpare
-// of the tile's; the others, and every particle of a component whose tile holds a NaN or an infinity or
-// nothing above 2^-895, are evaluated in FP64 from global memory (eval_f64_global).  That choice depends on the coefficients and the position
-// alone, so every route to the evaluation gives the same bits.
+// The error of a fixed-point result is a few units of the tile's scale whatever the stencil holds (rms 0.7,
+// largest 2.5 for u), that of FP64 arithmetic a multiple of 2^-53 sum w |a| (rms 0.8 to 2.5 at order 4, 0.9 to
+// 4 at order 8, for smooth, white and steep coefficients; the gradients' sums, sum |w'| |a|, are no smaller).  So a component is taken
+// from the fixed form where sum w |a| is at least 2^53 units (fixed::contract gives a lower estimate); the
+// others, and every particle of a component whose tile holds a NaN or an infinity or nothing above 2^-895, are
+// evaluated in FP64 from global memory (eval_f64_thread, eval_f64_warp): the low flanks of steep or localised fields, under
+// 0.1 % of the particles in a turbulent one, 1 % in a single Fourier mode (its nodal planes).  That choice
+// depends on the coefficients and the position alone, so every route to the evaluation gives the same bits.
 // Order 2 stays in FP64: with eight nodes a component the conversion costs more than it saves (256^3, 10^6
 // particles, a call 0.48 ms in FP64, 0.50 ms in fixed point).
 // NC = 3: a thread takes a particle's components in turn; NC = 1 (items of up to 42 particles): a thread
 // takes one component of a particle, the axes' weights being shared: with the 30 particles a brick of the
 // case above three of the four warps would idle otherwise (2.99 ms).
-constexpr int kSpare = 6;
+constexpr unsigned kFixedSize = 1u << (53 - 34);       // 2^53 units in those of fixed::contract
 template <int ORD, int NC> constexpr int fixed_threads() { return NC == 3 && ORD >= 7 ? 192 : 128; }
 template <int ORD, typename TR, bool GRAD, int NC>
 __global__ void __launch_bounds__(fixed_threads<ORD, NC>(), ORD >= 7 ? 2 : (ORD <= 4 ? 4 : 3))
@@ -930,7 +1046,8 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
     constexpr int T = fixed_threads<ORD, NC>();
     if (blockIdx.x >= w.chunk[bg.NB]) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ unsigned s_top[3], s_any[3];
+    __shared__ unsigned s_top[3], s_any[3], s_left;
+    __shared__ unsigned short s_pair[3 * (NC == 3 ? kFixedLong : kFixedShort)];      // 3 particle + component
     const unsigned brick = w.item[blockIdx.x];
     const unsigned beg = w.offset[brick] + (blockIdx.x - w.chunk[brick]) * chunk_len;
     const unsigned n = min(chunk_len, w.offset[brick] + w.count[brick] - beg);
@@ -957,6 +1074,7 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
         }
     }
     if (threadIdx.x < 3) s_top[threadIdx.x] = s_any[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_left = 0;
     cp_async_wait_all();
     __syncthreads();
     if constexpr (ORD == 2) {
@@ -1040,18 +1158,17 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
     }
     __syncthreads();
     int4* ws = reinterpret_cast<int4*>(smem_raw + align_up(tile_bytes<ORD, double>()));
-    // components c0 .. c0 + NC - 1 of one particle; wx(j): the x weights of node j
-    auto evaluate = [&](const Rec<TR>& rc, int c0, auto wx, const fixed::Limbs (&wy)[ORD], const fixed::Limbs (&dwy)[ORD],
-                        const fixed::Limbs (&wz)[ORD], const fixed::Limbs (&dwz)[ORD]) {
+    // components c0 .. c0 + NC - 1 of the item's particle i; wx(j): the x weights of node j
+    auto evaluate = [&](const Rec<TR>& rc, unsigned i, int c0, auto wx, const fixed::Limbs (&wy)[ORD],
+                        const fixed::Limbs (&dwy)[ORD], const fixed::Limbs (&wz)[ORD], const fixed::Limbs (&dwz)[ORD]) {
         const int ax = (int)(rc.cell >> (2 * kAnchorBits)), ay = (int)((rc.cell >> kAnchorBits) & 1023u);
         const int az = (int)(rc.cell & 1023u);
         const size_t idx = rc.idx;
         const uint2* base = words + (ax - x0) * S::SX + (ay - y0) * S::SY + (az - z0);
-        unsigned left = 0;                               // components that the fixed form does not represent
 #pragma unroll 1
         for (int c = c0; c < c0 + NC; ++c) {
             long long f[4];
-            int size = 0;
+            unsigned size = 0;
             const uint2* tc = base + c * S::TS;
             fixed::contract<ORD, GRAD>(
                 [&](int jx, int jy, int jz) {
@@ -1060,8 +1177,12 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
                 },
                 wx, wy, dwy, wz, dwz, f, &size);
             const int emax = (int)(s_top[c] >> 20);
-            if (!s_any[c]) f[0] = f[1] = f[2] = f[3] = 0;            // a component that is zero in the whole tile
-            else if (emax < fixed::kMinExponent || emax == 2047 || size < (1 << (29 - kSpare))) left |= 1u << c;
+            if (!s_any[c]) {
+                f[0] = f[1] = f[2] = f[3] = 0;           // a component that is zero in the whole tile
+            } else if (emax < fixed::kMinExponent || emax == 2047 || size < kFixedSize) {
+                s_pair[atomicAdd(&s_left, 1u)] = (unsigned short)(3 * i + c);       // not held by the fixed form
+                continue;
+            }
             // V 2^(emax - 1081), in two exact steps (one of them may leave the normal range)
             const int k = emax - 1081, k1 = k / 2;
             const double s1 = __hiloint2double((1023 + k1) << 20, 0), s2 = __hiloint2double((1023 + k - k1) << 20, 0);
@@ -1069,20 +1190,6 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
             if (GRAD) {
 #pragma unroll
                 for (int e = 0; e < 3; ++e) out_grad[9 * idx + 3 * c + e] = (((double)f[1 + e] * s1) * s2) * dscale;
-            }
-        }
-        if (left) {
-#pragma unroll 1
-            for (int c = 0; c < 3; ++c) {
-                if (!(left >> c & 1u)) continue;
-                double r[4];
-                eval_f64_global<ORD, GRAD>(coef + (size_t)c * N * N * N, N, ax, ay, az, rc.t[0], rc.t[1], rc.t[2],
-                                           dscale, r);
-                out_u[3 * idx + c] = r[0];
-                if (GRAD) {
-#pragma unroll
-                    for (int e = 0; e < 3; ++e) out_grad[9 * idx + 3 * c + e] = r[1 + e];
-                }
             }
         }
     };
@@ -1108,16 +1215,17 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
                 ws[(a * ORD + j) * kFixedShort + q] = make_int4(wy[j].hi, wy[j].lo, dwy[j].hi, dwy[j].lo);
         }
         __syncthreads();
-        if (!on || !record_ok(rc)) return;
+        if (on && record_ok(rc)) {
 #pragma unroll
-        for (int j = 0; j < ORD; ++j) {
-            const int4 y = ws[(ORD + j) * kFixedShort + q], v = ws[(2 * ORD + j) * kFixedShort + q];
-            wy[j] = {y.x, y.y};
-            dwy[j] = {y.z, y.w};
-            wz[j] = {v.x, v.y};
-            dwz[j] = {v.z, v.w};
+            for (int j = 0; j < ORD; ++j) {
+                const int4 y = ws[(ORD + j) * kFixedShort + q], v = ws[(2 * ORD + j) * kFixedShort + q];
+                wy[j] = {y.x, y.y};
+                dwy[j] = {y.z, y.w};
+                wz[j] = {v.x, v.y};
+                dwz[j] = {v.z, v.w};
+            }
+            evaluate(rc, q, (int)a, [&](int j) { return ws[j * kFixedShort + q]; }, wy, dwy, wz, dwz);
         }
-        evaluate(rc, (int)a, [&](int j) { return ws[j * kFixedShort + q]; }, wy, dwy, wz, dwz);
     } else {
         for (unsigned i = threadIdx.x; i < n; i += T) {
             const Rec<TR> rc = w.s_rec[beg + i];
@@ -1128,8 +1236,22 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
                 ws[j * T + threadIdx.x] = make_int4(wy[j].hi, wy[j].lo, dwy[j].hi, dwy[j].lo);
             fixed::weights<ORD>(fixed_t(rc.t[1]), wy, dwy);
             fixed::weights<ORD>(fixed_t(rc.t[2]), wz, dwz);
-            evaluate(rc, 0, [&](int j) { return ws[j * T + threadIdx.x]; }, wy, dwy, wz, dwz);
+            evaluate(rc, i, 0, [&](int j) { return ws[j * T + threadIdx.x]; }, wy, dwy, wz, dwz);
         }
+    }
+    // those left over, in FP64: few of them a warp each, many a thread each (a warp's form takes 54 to 130 FP64
+    // instructions a pair, a thread's 340 to 1700 for up to 32 pairs)
+    __syncthreads();
+    const unsigned left = s_left;
+    const bool by_warp = left <= 8 * (T / 32);
+    for (unsigned e = by_warp ? threadIdx.x >> 5 : threadIdx.x; e < left; e += by_warp ? T / 32 : T) {
+        const unsigned pair = s_pair[e], i = pair / 3, c = pair - 3 * i;
+        const Rec<TR> rc = w.s_rec[beg + i];
+        const double* comp = coef + (size_t)c * N * N * N;
+        double* u = out_u + 3 * (size_t)rc.idx + c;
+        double* g = GRAD ? out_grad + 9 * (size_t)rc.idx + 3 * c : nullptr;
+        if (by_warp) eval_f64_warp<ORD, GRAD>(comp, N, rc.cell, rc.t[0], rc.t[1], rc.t[2], dscale, u, g);
+        else eval_f64_thread<ORD, GRAD>(comp, N, rc.cell, rc.t[0], rc.t[1], rc.t[2], dscale, u, g);
     }
 }
 
