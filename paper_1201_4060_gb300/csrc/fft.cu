@@ -115,10 +115,14 @@ fft_x_prefilter(const typename Cx<R>::T* __restrict__ in, typename Cx<R>::T* __r
         for (int m = t; m < N; m += T) ftw[m] = twf[m];
         LineScale scale;
         if (stage_first_fixed<N, NL, T, NL>(fs, red, tops, ld, &scale)) {
-            stages_mid<Fx, N, NL, T, NL, radix_for(N)>(fs, ftw, 1);
-            stage_last<Fx, N, NL, T, NL, false>(fs, ftw, 1, [&](int q, int b, Fx v) {
-                if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
-            });
+            Steps steps = scale.steps();
+            stages_mid<Fx, N, NL, T, NL, radix_for(N)>(fs, ftw, 1, steps);
+            stage_last<Fx, N, NL, T, NL, false>(
+                fs, ftw, 1,
+                [&](int q, int b, Fx v) {
+                    if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
+                },
+                [&](int) { return steps; });
             return;
         }
         for (int m = t; m < N; m += T) tws[m] = tw[m];
@@ -395,10 +399,14 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                 done = stage_first_fixed<N, NLY, T, QY>(fbuf, red, tops, ld, &scale);
                 if (done) {
                     if (t == 0) prefetch_flag();
-                    stages_mid<Fx, N, NLY, T, QY, radix_for(N)>(fbuf, ftw, 1);
-                    stage_last<Fx, N, NLY, T, QY, false>(fbuf, ftw, 1, [&](int q, int b, Fx v) {
-                        if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
-                    });
+                    Steps steps = scale.steps();
+                    stages_mid<Fx, N, NLY, T, QY, radix_for(N)>(fbuf, ftw, 1, steps);
+                    stage_last<Fx, N, NLY, T, QY, false>(
+                        fbuf, ftw, 1,
+                        [&](int q, int b, Fx v) {
+                            if (col) st(q, b, make_double2(scale.out(v.x), scale.out(v.y)));
+                        },
+                        [&](int) { return steps; });
                 } else {
                     fp64_twiddles();
                 }
@@ -468,14 +476,15 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
             auto st = [&](int m, int b, V z) { store_pair<OutT, V>(dst + (long long)b * N + 2 * m, z); };
             bool done = false;
             if constexpr (FIXED) {
-                // scale of each row (z = E + i O: at most 1 + sqrt 2 times the norms of its two modes, each of
-                // which two z share), the row's modes in fixed point in place, then the stages
+                // scale of each row (z = a (1 + i w) + conj c (1 - i w) of its two modes, |1 + i w| + |1 - i w| <=
+                // 2 sqrt 2, and the two z that share them sum to at most that times |a| + |c|), the row's modes
+                // in fixed point in place, then the stages
                 constexpr int NT = T / NR;              // threads of a row
                 static_assert(T % NR == 0, "whole rows");
                 const int zb = t % NR;
                 V* row = raw + zb * RP;
                 LineScale scale;
-                done = line_scale<NR, T>(
+                done = line_scale<M, NR, T>(
                     [&](auto f) {
                         for (int k = t / NR; k <= kmax; k += NT) {
                             const V a = row[k];
@@ -483,7 +492,7 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                             f((unsigned)__double2hiint(a.y), (unsigned)__double2loint(a.y));
                         }
                     },
-                    5, red, tops, &scale);
+                    3, 2, red, tops, &scale);
                 if (done) {
                     for (int k = t / NR; k <= kmax; k += NT) {
                         const V a = row[k];
@@ -502,11 +511,15 @@ fft_yz_fused(const typename Cx<R>::T* __restrict__ w, OutT* __restrict__ out, ty
                         return {E.x - O.y, E.y + O.x};
                     };
                     stage_first<Fx, M, NR, T, QZ, true>(fbuf, ldf);
-                    stages_mid<Fx, M, NR, T, QZ, radix_for(M)>(fbuf, ftw, 2);
-                    stage_last<Fx, M, NR, T, QZ, true>(fbuf, ftw, 2, [&](int m, int b, Fx z) {
-                        const LineScale sb(tops[b]);
-                        st(m, b, make_double2(sb.out(z.x), sb.out(z.y)));
-                    });
+                    stages_mid<Fx, M, NR, T, QZ, radix_for(M)>(fbuf, ftw, 2, scale.steps());
+                    constexpr int taken = steps_between(M, radix_for(M), ns_last(M));
+                    stage_last<Fx, M, NR, T, QZ, true>(
+                        fbuf, ftw, 2,
+                        [&](int m, int b, Fx z) {
+                            const LineScale sb(tops[b]);
+                            st(m, b, make_double2(sb.out(z.x), sb.out(z.y)));
+                        },
+                        [&](int b) { return LineScale(tops[b]).steps_after(taken); });
                 } else {
                     fp64_twiddles();
                 }

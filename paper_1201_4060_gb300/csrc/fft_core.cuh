@@ -25,8 +25,14 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
 template <typename R> __device__ __forceinline__ R mul_sqrt_half(R v) { return v * (R)0.70710678118654752440084436210485; }
 template <typename R> __device__ __forceinline__ R mul_half_sqrt3(R v) { return v * (R)0.86602540378443864676372317075294; }
 template <typename R> __device__ __forceinline__ R sub_half(R a, R s) { return a - (R)0.5 * s; }
-__device__ __forceinline__ float2 twiddled(float2 a, float2 w) { return cmul(a, w); }
-__device__ __forceinline__ double2 twiddled(double2 a, double2 w) { return cmul(a, w); }
+// What a stage divides its input by (fixed point: a power of two, fft_fixed.cuh; else nothing), one step a stage.
+struct NoStep {};
+struct NoSteps {
+    template <int RADIX> __device__ __forceinline__ NoStep next() { return {}; }
+};
+template <typename V> __device__ __forceinline__ V rescaled(V a, NoStep) { return a; }
+__device__ __forceinline__ float2 twiddled(float2 a, float2 w, NoStep) { return cmul(a, w); }
+__device__ __forceinline__ double2 twiddled(double2 a, double2 w, NoStep) { return cmul(a, w); }
 template <typename V> __device__ __forceinline__ V cmuli(V a) { return mk<V>(-a.y, a.x); }  // a * (+i)
 
 // Inverse DFTs (exponent +2 pi i n k / R) in registers.
@@ -81,12 +87,13 @@ template <int R, typename V> __device__ __forceinline__ void butterfly(V* v) {
 // Butterfly j of a line reads positions j + r L/R, multiplies by
 // exp(2 pi i r (j mod NS) / (NS R)), and writes positions
 // (j / NS) NS R + (j mod NS) + r NS.  All reads finish before any write.
-template <typename V, int L, int NLINES, int T, int RADIX, int NS, int QS, typename W>
-__device__ __forceinline__ void stage(V* s, const W* tw, int twstride) {
+template <typename V, int L, int NLINES, int T, int RADIX, int NS, int QS, typename W, typename Steps = NoSteps>
+__device__ __forceinline__ void stage(V* s, const W* tw, int twstride, Steps&& steps = Steps()) {
     constexpr int NB = (L / RADIX) * NLINES;
     constexpr int BPT = (NB + T - 1) / T;
     V v[BPT][RADIX];
     const int t = threadIdx.x;
+    const auto step = steps.template next<RADIX>();
 #pragma unroll
     for (int i = 0; i < BPT; ++i) {
         const int u = t + i * T;
@@ -94,9 +101,9 @@ __device__ __forceinline__ void stage(V* s, const W* tw, int twstride) {
             const int b = u % NLINES, j = u / NLINES, k = j % NS;
 #pragma unroll
             for (int r = 0; r < RADIX; ++r) {
-                V a = s[(j + r * (L / RADIX)) * QS + b];
-                if (NS > 1 && r > 0) a = twiddled(a, tw[(r * k * (L / (NS * RADIX))) * twstride]);
-                v[i][r] = a;
+                const V a = s[(j + r * (L / RADIX)) * QS + b];
+                v[i][r] = (NS > 1 && r > 0) ? twiddled(a, tw[(r * k * (L / (NS * RADIX))) * twstride], step)
+                                            : rescaled(a, step);
             }
             butterfly<RADIX>(v[i]);
         }
@@ -169,21 +176,24 @@ __device__ __forceinline__ void stage_first(V* s, Ld ld) {
 }
 
 // Stages after the first, up to (not including) the last.
-template <typename V, int L, int NLINES, int T, int QS, int NS, typename W>
-__device__ __forceinline__ void stages_mid(V* s, const W* tw, int twstride) {
+template <typename V, int L, int NLINES, int T, int QS, int NS, typename W, typename Steps = NoSteps>
+__device__ __forceinline__ void stages_mid(V* s, const W* tw, int twstride, Steps&& steps = Steps()) {
     if constexpr (NS < ns_last(L)) {
         constexpr int RADIX = radix_for(L / NS);
-        stage<V, L, NLINES, T, RADIX, NS, QS>(s, tw, twstride);
-        stages_mid<V, L, NLINES, T, QS, NS * RADIX>(s, tw, twstride);
+        stage<V, L, NLINES, T, RADIX, NS, QS>(s, tw, twstride, steps);
+        stages_mid<V, L, NLINES, T, QS, NS * RADIX>(s, tw, twstride, steps);
     }
 }
 
 // Last stage (NS = L / R): butterfly j reads positions j + r NS, twiddles by
 // exp(2 pi i r j / L), and hands output position j + r NS of line b to st.
 // Consecutive threads take consecutive lines (JFAST = false) or consecutive
-// butterflies of one line (JFAST = true: stores along a line coalesce).
-template <typename V, int L, int NLINES, int T, int QS, bool JFAST, typename W, typename St>
-__device__ __forceinline__ void stage_last(const V* s, const W* tw, int twstride, St st) {
+// butterflies of one line (JFAST = true: stores along a line coalesce).  steps_of(b): line b's steps, at this stage.
+struct NoStepsOf {
+    __device__ __forceinline__ NoSteps operator()(int) const { return {}; }
+};
+template <typename V, int L, int NLINES, int T, int QS, bool JFAST, typename W, typename St, typename StepsOf = NoStepsOf>
+__device__ __forceinline__ void stage_last(const V* s, const W* tw, int twstride, St st, StepsOf steps_of = StepsOf()) {
     constexpr int NS = ns_last(L);
     constexpr int RADIX = L / NS;
     constexpr int NB = NS * NLINES;
@@ -194,12 +204,12 @@ __device__ __forceinline__ void stage_last(const V* s, const W* tw, int twstride
         const int u = t + i * T;
         if (NB % T == 0 || u < NB) {
             const int b = JFAST ? u / NS : u % NLINES, j = JFAST ? u % NS : u / NLINES;
+            const auto step = steps_of(b).template next<RADIX>();
             V v[RADIX];
 #pragma unroll
             for (int r = 0; r < RADIX; ++r) {
-                V a = s[(j + r * NS) * QS + b];
-                if (r > 0) a = twiddled(a, tw[(r * j) * twstride]);
-                v[r] = a;
+                const V a = s[(j + r * NS) * QS + b];
+                v[r] = r > 0 ? twiddled(a, tw[(r * j) * twstride], step) : rescaled(a, step);
             }
             butterfly<RADIX>(v);
 #pragma unroll
