@@ -2,15 +2,16 @@
 //
 // GB300 sustains 527 G FP64 operations a second (1.7 per clock per SM; measured, fma or add alike) but
 // 9000 G 32 x 32 -> 64-bit integer multiply-adds.  The stencil contraction of an FP64 plan is therefore
-// done on integers: a number v is held as the integer V = v 2^60 (weights) or v 2^(59 - E) (values, E the
-// exponent of the largest one of a tile), in two limbs
+// done on integers: a number v is held as the integer V = v 2^60 (weights) or v 2^(B - E) (values, 2^E the
+// power of two above the largest one of a tile), rounded to nearest, in two limbs
 //     V = hi 2^30 + lo,  lo in [-2^29, 2^29),
 // and a product sum  sum a b / 2^60  as  H + M 2^-30  with
 //     H = sum a.hi b.hi,  M = sum (a.hi b.lo + a.lo b.hi)
 // in 64-bit accumulators: three multiply-adds a term.  The omitted lo lo terms are below 2^-2 of the last
-// place each.  Bounds that keep every accumulator inside 63 bits, for up to 8 terms: weights |b| <= 2^60
-// with sum |b| <= 2 2^60 (node weights are non-negative and sum to one; derivative weights are a difference
-// of two such sets), values |a| <= 2^60: |H| <= 2^61, |M| <= 8 2^30 2^29 + 2 2^30 2^29 < 2^63.
+// place each.  Bounds that keep every accumulator inside 63 bits and every limb inside 31: weights |b| <= 2^60,
+// node weights non-negative with sum 1, derivative weights with sum |b| <= D: 2 at order 3, at most 1.5 from order 4
+// on.  Values |a| <= 2^B, sums after the derivative weights <= D 2^B: with B = 60 from order 4 on |hi| <= 1.5 2^30 and, for
+// up to 8 terms, |H| <= 1.5 2^60, |M| <= 8 (1.5 2^30) 2^29 + 2^29 (1.5 2^30) < 2^63; B = 59 at order 3.
 #pragma once
 
 namespace bs {
@@ -115,16 +116,19 @@ template <int n> BS_HD void weights(long long T, Limbs (&w)[n], Limbs (&dw)[n]) 
 
 BS_HD int exponent_bits(unsigned hi32) { return (int)((hi32 >> 20) & 0x7ffu); }
 
-// The fixed value, rounded down, of the double with words hi32, lo32 when the tile's largest biased
-// exponent is emax: v 2^(1081 - emax), |result| <= 2^59.  emax >= kMinExponent: zeros and subnormals, whose
-// implicit significand bit is not zeroed here, are then shifted out (to 0 or -1).
+// Bits of a tile's largest value.
+template <int n> constexpr int value_bits() { return n >= 4 ? 60 : 59; }
+
+// The fixed value, rounded to nearest, of the double with words hi32, lo32 when the tile's largest biased
+// exponent is emax: v 2^(1022 + bits - emax), |result| <= 2^bits.  emax >= kMinExponent: zeros and subnormals, whose
+// implicit significand bit is not zeroed here, are then shifted out.
 constexpr int kMinExponent = 128;
-BS_HD long long from_double(unsigned hi32, unsigned lo32, int emax) {
-    const int sh = emax - exponent_bits(hi32) + 4;       // from a significand of 63 bits
+BS_HD long long from_double(unsigned hi32, unsigned lo32, int emax, int bits) {
+    const int sh = emax - exponent_bits(hi32) + 62 - bits;   // from a significand of 63 bits; one less than the shift
     const long long m = (long long)(((unsigned long long)((hi32 & 0xfffffu) | 0x100000u) << 42) |
                                     ((unsigned long long)lo32 << 10));
     const long long sign = (long long)((int)hi32 >> 31);
-    return ((m ^ sign) - sign) >> (sh < 63 ? sh : 63);
+    return ((((m ^ sign) - sign) >> (sh < 63 ? sh : 63)) + 1) >> 1;
 }
 
 BS_HD unsigned mul_hi(unsigned a, unsigned b) { return (unsigned)(((unsigned long long)a * b) >> 32); }

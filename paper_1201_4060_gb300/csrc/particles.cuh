@@ -1022,14 +1022,15 @@ __device__ __noinline__ void eval_f64_warp(const double* __restrict__ comp, int 
 // derivatives are integer multiply-adds, and only the twelve results are FP64 again.  Bound: integer issue.
 // The FP64 pipe took 1900 operations a particle at order 6: 5.36 ms for 10^6 particles on 256^3; the fixed
 // form's 5100 wide multiply-adds, with the tile's conversion (216 values a particle there), take 1.72 ms.
-// The error of a fixed-point result is a few units of the tile's scale whatever the stencil holds (rms 0.7,
-// largest 2.5 for u), that of FP64 arithmetic a multiple of 2^-53 sum w |a| (rms 0.8 to 2.5 at order 4, 0.9 to
-// 4 at order 8, for smooth, white and steep coefficients; the gradients' sums, sum |w'| |a|, are no smaller).  So a component is taken
-// from the fixed form where sum w |a| is at least 2^53 units (fixed::contract gives a lower estimate); the
-// others, and every particle of a component whose tile holds a NaN or an infinity or nothing above 2^-895, are
-// evaluated in FP64 from global memory (eval_f64_thread, eval_f64_warp): the low flanks of steep or localised fields, under
-// 0.1 % of the particles in a turbulent one, 1 % in a single Fourier mode (its nodal planes).  That choice
-// depends on the coefficients and the position alone, so every route to the evaluation gives the same bits.
+// The error of a fixed-point result is a unit or two whatever the stencil holds (rms 0.7, largest 2.5 for u; a unit is
+// 2^-59 to 2^-60 of the tile's largest value from order 4 on, twice that at order 3), that of FP64 arithmetic a
+// multiple of 2^-53 sum w |a| (rms 0.8 to 2.5 at order 4, 0.9 to 4 at order 8, for smooth, white and steep
+// coefficients; the sums that the gradients are rounded against are no smaller).  So a component is taken from the
+// fixed form where sum w |a| is at least 2^53 units (fixed::contract gives a lower estimate); the others, and every
+// particle of a component whose tile holds a NaN or an infinity or nothing above 2^-895, are evaluated in FP64
+// from global memory (eval_f64_thread, eval_f64_warp): the low flanks of steep or localised fields, one particle
+// in 10^4 or fewer of a turbulent one, 1 % in a single Fourier mode (its nodal planes).  That choice depends on the
+// coefficients and the position alone, so every route to the evaluation gives the same bits.
 // Order 2 stays in FP64: with eight nodes a component the conversion costs more than it saves (256^3, 10^6
 // particles, a call 0.48 ms in FP64, 0.50 ms in fixed point).
 // NC = 3: a thread takes a particle's components in turn; NC = 1 (items of up to 42 particles): a thread
@@ -1043,7 +1044,7 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
              double* __restrict__ out_u, double* __restrict__ out_grad, double dscale,
              unsigned long long* __restrict__ status) {
     using S = Shape<double, ORD>;
-    constexpr int T = fixed_threads<ORD, NC>();
+    constexpr int T = fixed_threads<ORD, NC>(), kBits = fixed::value_bits<ORD>();
     if (blockIdx.x >= w.chunk[bg.NB]) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned s_top[3], s_any[3], s_left;
@@ -1152,7 +1153,7 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
         const int emax = (int)(s_top[c] >> 20);
         for (int k = threadIdx.x; k < S::TS; k += T) {
             const uint2 d = words[c * S::TS + k];
-            const fixed::Limbs l = fixed::limbs(fixed::from_double(d.y, d.x, emax));
+            const fixed::Limbs l = fixed::limbs(fixed::from_double(d.y, d.x, emax, kBits));
             words[c * S::TS + k] = make_uint2((unsigned)l.lo, (unsigned)l.hi);
         }
     }
@@ -1183,8 +1184,8 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
                 s_pair[atomicAdd(&s_left, 1u)] = (unsigned short)(3 * i + c);       // not held by the fixed form
                 continue;
             }
-            // V 2^(emax - 1081), in two exact steps (one of them may leave the normal range)
-            const int k = emax - 1081, k1 = k / 2;
+            // V 2^(emax - 1022 - kBits), in two exact steps (one of them may leave the normal range)
+            const int k = emax - 1022 - kBits, k1 = k / 2;
             const double s1 = __hiloint2double((1023 + k1) << 20, 0), s2 = __hiloint2double((1023 + k - k1) << 20, 0);
             out_u[3 * idx + c] = ((double)f[0] * s1) * s2;
             if (GRAD) {
