@@ -403,19 +403,23 @@ inline unsigned grid_for(long long P, int threads) {
 // copies bound the placement), 455 + 465 -> 55 + 76 us clustered on 128^3 (704 bricks, whose counters the
 // warps queued for).  Else an atomic a particle and pass: at 512^3 (44032 bricks, 2^24 particles) places
 // returned by the count's atomics made the step 1.5 % slower; at 5632 bricks and 10^6 particles the runs
-// (3328) gain nothing.
+// (3328) gain nothing.  Never for sorted input: a warp's particles share a brick or two, one atomic each, and
+// nothing is placed afterwards (FP32, 64^3 in brick order, histogram / warp: 2000 particles, order 4, 34.6 / 29.3 us a
+// call; 50000 41.7 / 36.3; 10^6, order 2, 111 / 103).
 template <typename TR, bool SORTED, typename OT>
 bool launch_bin(bspline_plan_s* p, const double* x, int64_t P, const BrickGrid& g, const Ws<TR>& w, OT* ou, OT* og,
                 unsigned grid, unsigned long long* status, cudaStream_t st) {
     const double scale = (double)p->N / p->L;
     const unsigned run = (unsigned)std::min<long long>(8192, std::max<long long>(1024, (P / (2 * p->sms) + 255) / 256 * 256));
-    if (g.NB <= std::max(run, 4096u)) {
-        const size_t sm = sizeof(unsigned) * (g.NB + 1 + run);
-        auto k = bin_kernel<TR, SORTED, true, OT>;
-        if (set_smem(k, sm) == BSPLINE_OK) {
-            const unsigned runs = (unsigned)((P + run - 1) / run);
-            k<<<std::min(runs, grid), 256, sm, st>>>(x, P, p->N, scale, p->order, g, w, status, run, ou, og);
-            return true;
+    if constexpr (!SORTED) {
+        if (g.NB <= std::max(run, 4096u)) {
+            const size_t sm = sizeof(unsigned) * (g.NB + 1 + run);
+            auto k = bin_kernel<TR, false, true, OT>;
+            if (set_smem(k, sm) == BSPLINE_OK) {
+                const unsigned runs = (unsigned)((P + run - 1) / run);
+                k<<<std::min(runs, grid), 256, sm, st>>>(x, P, p->N, scale, p->order, g, w, status, run, ou, og);
+                return true;
+            }
         }
     }
     bin_kernel<TR, SORTED, false, OT><<<grid, 256, 0, st>>>(x, P, p->N, scale, p->order, g, w, status, 0u, ou, og);
