@@ -479,10 +479,10 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     const unsigned NB = g.NB;
     Ws<TR> w;
     const unsigned len = item_particles(p->dtype, P, NB);
-    const size_t need = carve<TR>(&w, nullptr, NB, P, len);
+    const size_t need = carve<TR>(&w, nullptr, NB, P, shortest_item(p->dtype));
     int rc = p->pws.grow(need);
     if (rc) return rc;
-    carve<TR>(&w, p->pws.ptr, NB, P, len);
+    carve<TR>(&w, p->pws.ptr, NB, P, shortest_item(p->dtype));
     const cudaStream_t main_stream = p->stream;
     cudaStream_t st = sort_stream ? sort_stream : main_stream;
     p->stream = st;                                     // stage timers follow the sort's stream
@@ -557,7 +557,7 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const unsigned NB = g.NB;
     Ws<TR> w;
     const unsigned len = item_particles(p->dtype, P, NB);
-    carve<TR>(&w, ws, NB, P, len);
+    carve<TR>(&w, ws, NB, P, shortest_item(p->dtype));
     cudaStream_t st = p->stream;
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (NB + 2), st)) != cudaSuccess) return set_cuda_error(e);
@@ -711,10 +711,10 @@ size_t interp_workspace_bytes(const bspline_plan_s* p, int64_t P) {
     const unsigned NB = g.NB;
     if (p->dtype == BSPLINE_F64) {
         Ws<double> w;
-        return carve<double>(&w, nullptr, NB, P, item_particles(p->dtype, P, NB));
+        return carve<double>(&w, nullptr, NB, P, shortest_item(p->dtype));
     }
     Ws<float> w;
-    return carve<float>(&w, nullptr, NB, P, item_particles(p->dtype, P, NB));
+    return carve<float>(&w, nullptr, NB, P, shortest_item(p->dtype));
 }
 
 int launch_interp_split(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u,

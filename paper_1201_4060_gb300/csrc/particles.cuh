@@ -50,6 +50,10 @@ inline unsigned item_particles(int dtype, int64_t P, unsigned NB) {
     return dtype != BSPLINE_F64 ? kChunk : (P >= 256LL * NB ? kFixedLong : kFixedShort);
 }
 
+// The shortest items of a type: what the workspace holds places for, so that a call of fewer particles never needs a
+// larger one (131071 particles on 64^3 take items of 42, 131072 items of 512).
+constexpr unsigned shortest_item(int dtype) { return dtype == BSPLINE_F64 ? kFixedShort : kChunk; }
+
 template <typename TR> struct Ws {
     unsigned* count;    // [NB + 2]  particles per brick; slot NB = invalid positions; NB + 1 = *unsorted
     unsigned* unsorted; // nonzero if positions passed as sorted were not in brick order (count pass)
@@ -58,14 +62,14 @@ template <typename TR> struct Ws {
     unsigned* cursor;   // [NB + 1]  next free sorted slot of each brick (starts at offset), without ranks
     unsigned* rank;     // [P]       each particle's place within its brick (count pass by histograms)
     unsigned* chunk;    // [NB + 1]  exclusive prefix sum of ceil(count / chunk_len): first work item of a brick
-    unsigned* item;     // [NB + ceil(P / chunk_len)]  brick of each work item (the first chunk[NB] are set)
+    unsigned* item;     // [NB + ceil(P / shortest)]  brick of each work item (the first chunk[NB] are set)
     long long P;        // particles
     Rec<TR>* s_rec;     // [P]       located records sorted by brick
 };
 
 constexpr size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
-template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t P, unsigned chunk_len = kChunk) {
+template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t P, unsigned shortest = kChunk) {
     size_t off = 0;
     auto take = [&](size_t bytes) {
         void* ptr = base ? (void*)((char*)base + off) : nullptr;
@@ -79,7 +83,7 @@ template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t 
     w->cursor = (unsigned*)take(sizeof(unsigned) * (NB + 1));
     w->rank = (unsigned*)take(sizeof(unsigned) * P);
     w->chunk = (unsigned*)take(sizeof(unsigned) * (NB + 1));
-    w->item = (unsigned*)take(sizeof(unsigned) * (NB + (P + chunk_len - 1) / chunk_len));
+    w->item = (unsigned*)take(sizeof(unsigned) * (NB + (P + shortest - 1) / shortest));
     w->s_rec = (Rec<TR>*)take(sizeof(Rec<TR>) * P);
     return off;
 }
