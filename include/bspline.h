@@ -156,10 +156,13 @@ int bspline_plan_set_gather_split(bspline_plan_t plan, unsigned direct_below);
  * (device buffers as for bspline_interp, out_grad NULL for u only) with the
  * split at 0, 8, 32, 128, 512 and "every brick direct", sets the fastest on
  * the plan and returns it in *split_out and its time per call in *ms_out
- * (either may be NULL).  out_u and out_grad are scratch: on return they
+ * (either may be NULL).  Where these P particles are few enough not to be
+ * sorted, "every brick direct" times that route, and if it is the fastest
+ * BSPLINE_GATHER_SPLIT_AUTO is set, which takes it for such calls only.
+ * out_u and out_grad are scratch: on return they
  * hold the result of the last timed call.  If the environment variable
  * BSPLINE_AUTOTUNE_CACHE names a file, a choice recorded there for the same
- * (GPU name, N, order, dtype, ceil(log2 P)) is applied without timing
+ * (GPU name, N, order, dtype, ceil(log2 P), sorted or not) is applied without timing
  * (*ms_out = 0), and a new choice is appended to it as one JSON line.
  * Synchronises the plan's stream. */
 int bspline_plan_autotune(bspline_plan_t plan, const void* coeffs, const double* x, int64_t P, void* out_u,

@@ -513,7 +513,15 @@ int bspline_plan_autotune(bspline_plan_t plan, const void* coeffs, const double*
     DeviceGuard g(plan->device);
     if (!g.ok) return BSPLINE_ERR_CUDA;
     const int flags = out_grad ? 0 : BSPLINE_INTERP_NO_GRAD;
-    // cache key: GPU name, grid, order, dtype, particle count rounded up to a power of two
+    // A call that AUTO evaluates without a sort times that route as "every brick direct"; set is AUTO then, so that
+    // another count, or a call beside a transform, which was not timed, keeps the rule instead of sorting into the
+    // direct gather.
+    const unsigned before = plan->direct_below;
+    plan->direct_below = BSPLINE_GATHER_SPLIT_AUTO;
+    const bool unsorted = !interp_sorts(plan, P, flags);
+    plan->direct_below = before;
+    const auto to_set = [&](unsigned split) { return unsorted && split == 0xffffffffu ? BSPLINE_GATHER_SPLIT_AUTO : split; };
+    // cache key: GPU name, grid, order, dtype, particle count rounded up to a power of two, route
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, plan->device);
     if (e != cudaSuccess) return set_cuda_error(e);
@@ -521,7 +529,8 @@ int bspline_plan_autotune(bspline_plan_t plan, const void* coeffs, const double*
     while (plog2 < 62 && (1LL << plog2) < (long long)P) ++plog2;
     static const char* kDtype[] = {"f64", "f32", "bf16"};
     char key[384];
-    std::snprintf(key, sizeof key, "%s|N%d|o%d|%s|p2^%d", prop.name, plan->N, plan->order, kDtype[plan->dtype], plog2);
+    std::snprintf(key, sizeof key, "%s|N%d|o%d|%s|p2^%d|%s", prop.name, plan->N, plan->order, kDtype[plan->dtype], plog2,
+                  unsorted ? "unsorted" : "sorted");
     const char* path = std::getenv("BSPLINE_AUTOTUNE_CACHE");
     if (path && *path) {
         if (FILE* f = std::fopen(path, "r")) {
@@ -537,7 +546,7 @@ int bspline_plan_autotune(bspline_plan_t plan, const void* coeffs, const double*
             }
             std::fclose(f);
             if (found) {
-                plan->direct_below = split;
+                plan->direct_below = to_set(split);
                 if (split_out) *split_out = split;
                 if (ms_out) *ms_out = 0.0;
                 return BSPLINE_OK;
@@ -570,7 +579,7 @@ int bspline_plan_autotune(bspline_plan_t plan, const void* coeffs, const double*
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    plan->direct_below = best;
+    plan->direct_below = rc ? before : to_set(best);
     if (rc) return rc;
     if (split_out) *split_out = best;
     if (ms_out) *ms_out = best_ms / 3.0;

@@ -164,7 +164,8 @@ int launch_coeffs_fields(const bspline_plan_s* p, int F, const void* const* in_f
 size_t interp_workspace_bytes(const bspline_plan_s* p, int64_t P);
 int launch_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u,
                   void* out_grad, int flags);
-// Whether an evaluation beside a transform sorts its particles (few of them are evaluated in the caller's order).
+// Whether an evaluation sorts its particles (few of them are evaluated in the caller's order): alone, beside a transform.
+bool interp_sorts(const bspline_plan_s* p, int64_t P, int flags);
 bool eval_sorts(const bspline_plan_s* p, int64_t P, int flags);
 // The same, with the sort on sort_stream (recording `sorted` there) and the
 // gather on the plan's stream once `sorted` has been reached.

@@ -731,6 +731,7 @@ int launch_interp_split(bspline_plan_s* p, const void* coeffs, const double* x, 
     return BSPLINE_ERR_INVALID_ARG;
 }
 
+bool interp_sorts(const bspline_plan_s* p, int64_t P, int flags) { return !unsorted_call(p, P, flags, false); }
 bool eval_sorts(const bspline_plan_s* p, int64_t P, int flags) { return !unsorted_call(p, P, flags, true); }
 
 int launch_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u, void* out_grad,

@@ -1,8 +1,14 @@
-"""Rules that pick a route by a call's size, from outside: workspaces that smaller calls never outgrow."""
+"""Rules that pick a route by a call's size, from outside: workspaces that smaller calls never outgrow, the autotuner's
+choice and its cache for calls with and without a sort, and the sorted route at sizes whose calls AUTO does not sort."""
+import math
+
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+L = 2.0 * math.pi
+ALL_DIRECT = 2 ** 32 - 1
 
 
 @pytest.fixture(scope="module")
@@ -11,6 +17,17 @@ def B():
     _build.build()
     from paper_1201_4060_gb300 import bspline
     return bspline
+
+
+def positions(P, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand((P, 3), generator=g, dtype=torch.float64, device="cuda") * L
+
+
+def field(plan, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    N = plan.N
+    return torch.randn((3, N, N, N // 2 + 1), generator=g, dtype=plan.uhat_dtype, device="cuda")
 
 
 @pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
@@ -24,4 +41,90 @@ def test_workspace_never_shrinks_with_more_particles(B, dtype, N):
                                      300000) for d in (-1, 0, 1) if p + d > 0})
     sizes = [plan.workspace_bytes(p) for p in counts]
     assert sizes == sorted(sizes)
+    plan.close()
+
+
+def key(N, order, P, route):
+    return (f"{torch.cuda.get_device_properties(0).name}|N{N}|o{order}|f32|p2^{max(P - 1, 1).bit_length()}"
+            + (f"|{route}" if route else ""))
+
+
+@pytest.mark.parametrize("route", ["", "unsorted"])
+def test_all_direct_timed_without_a_sort_is_not_taken_for_a_sorted_call(B, route, tmp_path, monkeypatch):
+    """Order 6 sorts from 58255 particles on: a choice of "every brick direct" that was timed for fewer of the same
+    power of two, without a sort, says nothing about 60000."""
+    N, order, P = 32, 6, 60000
+    cache = tmp_path / "autotune.jsonl"
+    cache.write_text('{"key": "%s", "direct_below": %d, "ms": 0.0100}\n' % (key(N, order, P, route), ALL_DIRECT))
+    monkeypatch.setenv("BSPLINE_AUTOTUNE_CACHE", str(cache))
+    plan = B.Plan(N, order, "f32")
+    coef = plan.coeffs(field(plan, 1))
+    _, ms = plan.autotune(coef, positions(P, 2))
+    assert ms > 0                                        # timed, not taken from the file
+    plan.close()
+
+
+def test_all_direct_chosen_without_a_sort_leaves_larger_calls_to_the_rule(B, tmp_path, monkeypatch):
+    """A plan tuned on few particles: more of them, or a call beside a transform, are not sorted into the direct
+    gather (whose stage is then timed), which was not what was timed."""
+    N, order, P = 32, 6, 40000                           # beside a transform 14563 particles are sorted already
+    cache = tmp_path / "autotune.jsonl"
+    cache.write_text('{"key": "%s", "direct_below": %d, "ms": 0.0100}\n' % (key(N, order, P, "unsorted"), ALL_DIRECT))
+    monkeypatch.setenv("BSPLINE_AUTOTUNE_CACHE", str(cache))
+    plan = B.Plan(N, order, "f32")
+    u_hat = field(plan, 1)
+    coef = plan.coeffs(u_hat)
+    x = positions(P, 2)
+    split, ms = plan.autotune(coef, x)
+    assert (split, ms) == (ALL_DIRECT, 0.0)
+    plan.set_timing(True)
+    for calls, direct in ((lambda: plan.interp(coef, x), 1), (lambda: plan.interp(coef, positions(100000, 3)), 0),
+                          (lambda: plan.eval(u_hat, x), 0)):
+        plan.stage_times()
+        calls()
+        assert plan.stage_times()["gather_direct"][1] == direct
+    plan.close()
+
+
+@pytest.mark.parametrize("N", [768, 1024])
+def test_largest_grids_sorted_and_unsorted_agree(B, N):
+    """The sort, the scan of the most bricks and the staged gather, against the call that AUTO does not sort."""
+    order, P = 6, 4096
+    plan = B.Plan(N, order, "f32")
+    g = torch.Generator(device="cuda").manual_seed(N)
+    coef = torch.randn((3, N, N, N), generator=g, device="cuda")
+    x = positions(P, N)
+    x[:2000] = x[:2000] * 0.01 + 1.0                     # some bricks hold many
+    outs = []
+    for split in (B.GATHER_SPLIT_AUTO, 0, 16, ALL_DIRECT - 2):
+        plan.set_gather_split(split)
+        u, grad = plan.interp(coef, x)
+        assert plan.status() == 0
+        outs.append((u, grad))
+    for u, grad in outs[1:]:
+        assert torch.equal(u, outs[0][0]) and torch.equal(grad, outs[0][1])
+    plan.close()
+    del coef, outs
+    torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("split", [0, 32])
+def test_sort_beside_the_transform_agrees_with_the_unsorted_call(B, dtype, split):
+    """bspline_eval and bspline_run_host with the sort on the second stream, at sizes that AUTO does not sort."""
+    N, order, P = 32, 6, 5000
+    plan = B.Plan(N, order, dtype)
+    u_hat, x = field(plan, 3), positions(P, 4)
+    x[17, 1] = math.nan
+    coef, u, grad = plan.eval(u_hat, x)
+    assert plan.status() == 1
+    plan.set_gather_split(split)
+    coef2, u2, grad2 = plan.eval(u_hat, x)
+    assert plan.status() == 1
+    uh, xh = u_hat.cpu().pin_memory(), x.cpu().pin_memory()
+    uo, go = torch.empty((P, 3)).pin_memory(), torch.empty((P, 3, 3)).pin_memory()
+    plan.run_host(uh, xh, uo, go)
+    assert plan.status() == 1 and torch.equal(coef, coef2)
+    for a, b in ((u, u2), (grad, grad2), (u, uo.cuda()), (grad, go.cuda())):
+        assert torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0))
     plan.close()
