@@ -403,16 +403,19 @@ inline unsigned grid_for(long long P, int threads) {
 // copies bound the placement), 455 + 465 -> 55 + 76 us clustered on 128^3 (704 bricks, whose counters the
 // warps queued for).  Else an atomic a particle and pass: at 512^3 (44032 bricks, 2^24 particles) places
 // returned by the count's atomics made the step 1.5 % slower; at 5632 bricks and 10^6 particles the runs
-// (3328) gain nothing.  Never for sorted input: a warp's particles share a brick or two, one atomic each, and
-// nothing is placed afterwards (FP32, 64^3 in brick order, histogram / warp: 2000 particles, order 4, 34.6 / 29.3 us a
-// call; 50000 41.7 / 36.3; 10^6, order 2, 111 / 103).
+// (3328) gain nothing.  Few particles do not repay the zeroing and flushing of the bins (FP64 u at order 2, atomics /
+// histogram, us a call: 64 bricks, 4000 particles 30.2 / 33.1, 16000 37.2 / 35.5; 512 bricks, 16000 36.8 / 38.6, 64000
+// 58.5 / 49.3; 4096 bricks, 64000 54.6 / 63.0, 256000 109.6 / 110.3, 10^6 310 / 293).  Never for sorted input: a warp's
+// particles share a brick or two, one atomic each, and nothing is placed afterwards (FP32, 64^3 in brick order,
+// histogram / warp: 2000 particles, order 4, 34.6 / 29.3 us a call; 50000 41.7 / 36.3; 10^6, order 2, 111 / 103).
+constexpr long long kHistLeast = 12288, kHistPerBrick = 64;   // particles in all, particles a brick
 template <typename TR, bool SORTED, typename OT>
 bool launch_bin(bspline_plan_s* p, const double* x, int64_t P, const BrickGrid& g, const Ws<TR>& w, OT* ou, OT* og,
                 unsigned grid, unsigned long long* status, cudaStream_t st) {
     const double scale = (double)p->N / p->L;
     const unsigned run = (unsigned)std::min<long long>(8192, std::max<long long>(1024, (P / (2 * p->sms) + 255) / 256 * 256));
     if constexpr (!SORTED) {
-        if (g.NB <= std::max(run, 4096u)) {
+        if (g.NB <= std::max(run, 4096u) && P >= std::max(kHistLeast, kHistPerBrick * g.NB)) {
             const size_t sm = sizeof(unsigned) * (g.NB + 1 + run);
             auto k = bin_kernel<TR, false, true, OT>;
             if (set_smem(k, sm) == BSPLINE_OK) {

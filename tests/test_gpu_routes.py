@@ -128,3 +128,31 @@ def test_sort_beside_the_transform_agrees_with_the_unsorted_call(B, dtype, split
     for a, b in ((u, u2), (grad, grad2), (u, uo.cuda()), (grad, go.cuda())):
         assert torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0))
     plan.close()
+
+
+@pytest.mark.parametrize("dtype,N", [("f64", 32), ("f64", 64), ("f32", 64), ("bf16", 128)])
+def test_counting_by_runs_and_by_particles_agree(B, dtype, N):
+    """Both sides of the rule that counts particles by runs in shared memory (12288 of them, 64 a brick): every
+    particle is placed once, and its results are the same bits."""
+    order = 3
+    plan = B.Plan(N, order, dtype)
+    plan.set_gather_split(0)
+    bricks = (N // 8) ** 3 if dtype == "f64" else (N // 16) ** 2 * -(-N // 12)
+    edge = max(12288, 64 * bricks)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    real = torch.float64 if dtype == "f64" else torch.float32
+    coef = torch.randn((3, N, N, N), generator=g, dtype=real, device="cuda").to(plan.coef_dtype)
+    x = positions(edge + 1, N)
+    x[5, 2] = math.nan
+    x[edge // 2] = 1.0
+    outs = []
+    for P in (edge + 1, edge, edge - 1):
+        u, grad = plan.interp(coef, x[:P].contiguous())
+        assert plan.status() == 1
+        perm = plan.sort_order(x[:P].contiguous())
+        assert torch.equal(perm.sort().values.long(), torch.arange(P, device="cuda")) and int(perm[-1]) == 5
+        outs.append((u[:edge - 1], grad[:edge - 1]))
+    for u, grad in outs[1:]:
+        assert torch.equal(torch.nan_to_num(u, 7.0), torch.nan_to_num(outs[0][0], 7.0))
+        assert torch.equal(torch.nan_to_num(grad, 7.0), torch.nan_to_num(outs[0][1], 7.0))
+    plan.close()
