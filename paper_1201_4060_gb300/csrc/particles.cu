@@ -175,11 +175,11 @@ __device__ __forceinline__ unsigned warp_inclusive(unsigned v, unsigned lane) {
 }
 
 // SPLIT = false (below = 0: every brick dense) skips the sparse bookkeeping.
-// Bound: one CTA's latency per tile.  A thread takes kScanRun consecutive bricks (16-byte loads and
-// stores), the next tile's counts requested before this tile is scanned: 44032 bricks (512^3) in 6 tiles
-// instead of 43.
-constexpr unsigned kScanRun = 8;
-template <bool SPLIT>
+// Bound: one CTA's latency per tile.  A thread takes RUN consecutive bricks (4: 16-byte loads and stores), the next
+// tile's counts requested before this tile is scanned.  Measured with runs of 1 / 2 / 4 / 8: 96 bricks 6.2 / 6.4 / 7.6 /
+// 8.5 us, 5632 11.1 / 10.4 / 10.3 / 11.9, 18432 23.6 / 22.4 / 18.8 / 24.6, 44032 48 / 45 / 35 / 52: 1 where one tile of it
+// holds the bricks, else 4.
+template <bool SPLIT, unsigned RUN>
 __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__ count, unsigned* __restrict__ offset,
                                                     unsigned* __restrict__ cursor, unsigned* __restrict__ chunk,
                                                     unsigned* __restrict__ item, unsigned NB, unsigned below,
@@ -187,37 +187,36 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
     __shared__ unsigned wd[32], wsp[32], wc[32];
     const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned V = (unsigned)P - count[NB];           // valid particles
-    unsigned v[kScanRun], nx[kScanRun];
+    unsigned v[RUN], nx[RUN];
     auto load = [&](unsigned b0) {                        // the run's counts, zero beyond the bricks
-        const unsigned i = b0 + t * kScanRun;
-        if (i + kScanRun <= NB) {
-#pragma unroll
-            for (unsigned k = 0; k < kScanRun; k += 4) {
-                const uint4 q = *reinterpret_cast<const uint4*>(count + i + k);
-                nx[k] = q.x;
-                nx[k + 1] = q.y;
-                nx[k + 2] = q.z;
-                nx[k + 3] = q.w;
+        const unsigned i = b0 + t * RUN;
+        if constexpr (RUN == 4) {
+            if (i + RUN <= NB) {
+                const uint4 q = *reinterpret_cast<const uint4*>(count + i);
+                nx[0] = q.x;
+                nx[1] = q.y;
+                nx[2] = q.z;
+                nx[3] = q.w;
+                return;
             }
-        } else {
-#pragma unroll
-            for (unsigned k = 0; k < kScanRun; ++k) nx[k] = i + k < NB ? count[i + k] : 0u;
         }
+#pragma unroll
+        for (unsigned k = 0; k < RUN; ++k) nx[k] = i + k < NB ? count[i + k] : 0u;
     };
     unsigned cd = 0, cs = 0, cc = 0;                      // carries: dense, sparse, items
     // tiles of 1024 runs: sums of the runs, warp scans of those, then a scan of the 32 warp totals
     load(0);
-    for (unsigned b0 = 0; b0 < NB; b0 += 1024 * kScanRun) {
+    for (unsigned b0 = 0; b0 < NB; b0 += 1024 * RUN) {
         unsigned sd = 0, ss = 0, sc = 0;
 #pragma unroll
-        for (unsigned k = 0; k < kScanRun; ++k) {
+        for (unsigned k = 0; k < RUN; ++k) {
             v[k] = nx[k];
             const bool dense = !SPLIT || v[k] >= below;
             sd += dense ? v[k] : 0u;
             ss += dense ? 0u : v[k];
             sc += dense ? (v[k] + chunk_len - 1) / chunk_len : 0u;
         }
-        if (b0 + 1024 * kScanRun < NB) load(b0 + 1024 * kScanRun);
+        if (b0 + 1024 * RUN < NB) load(b0 + 1024 * RUN);
         const unsigned vd = warp_inclusive(sd, lane), vc = warp_inclusive(sc, lane);
         const unsigned vs = SPLIT ? warp_inclusive(ss, lane) : 0u;
         if (lane == 31) {
@@ -235,10 +234,10 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
         unsigned exd = cd + (warp ? wd[warp - 1] : 0u) + vd - sd;                 // exclusive
         unsigned exs = V - cs - (warp ? wsp[warp - 1] : 0u) - vs + ss;              // end of the run's segments
         unsigned exc = cc + (warp ? wc[warp - 1] : 0u) + vc - sc;
-        const unsigned i = b0 + t * kScanRun;
-        unsigned o[kScanRun], c[kScanRun];
+        const unsigned i = b0 + t * RUN;
+        unsigned o[RUN], c[RUN];
 #pragma unroll
-        for (unsigned k = 0; k < kScanRun; ++k) {
+        for (unsigned k = 0; k < RUN; ++k) {
             const bool dense = !SPLIT || v[k] >= below;
             exs -= dense ? 0u : v[k];
             o[k] = dense ? exd : exs;
@@ -248,17 +247,19 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
             exd += dense ? v[k] : 0u;
             exc += nc;
         }
-        if (i + kScanRun <= NB) {
-#pragma unroll
-            for (unsigned k = 0; k < kScanRun; k += 4) {
-                const uint4 a = make_uint4(o[k], o[k + 1], o[k + 2], o[k + 3]);
-                *reinterpret_cast<uint4*>(offset + i + k) = a;
-                *reinterpret_cast<uint4*>(cursor + i + k) = a;
-                *reinterpret_cast<uint4*>(chunk + i + k) = make_uint4(c[k], c[k + 1], c[k + 2], c[k + 3]);
+        bool stored = false;
+        if constexpr (RUN == 4) {
+            if (i + RUN <= NB) {
+                const uint4 a = make_uint4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<uint4*>(offset + i) = a;
+                *reinterpret_cast<uint4*>(cursor + i) = a;
+                *reinterpret_cast<uint4*>(chunk + i) = make_uint4(c[0], c[1], c[2], c[3]);
+                stored = true;
             }
-        } else {
+        }
+        if (!stored) {
 #pragma unroll
-            for (unsigned k = 0; k < kScanRun; ++k)
+            for (unsigned k = 0; k < RUN; ++k)
                 if (i + k < NB) {
                     offset[i + k] = o[k];
                     cursor[i + k] = o[k];
@@ -277,6 +278,13 @@ __global__ void __launch_bounds__(1024) scan_kernel(const unsigned* __restrict__
         offset[NB + 2] = cd;
         chunk[NB] = cc;
     }
+}
+
+template <typename TR>
+void launch_scan(const Ws<TR>& w, unsigned NB, unsigned below, unsigned chunk_len, long long P, cudaStream_t st) {
+    const auto k = NB <= 1024u ? (below ? scan_kernel<true, 1> : scan_kernel<false, 1>)
+                               : (below ? scan_kernel<true, 4> : scan_kernel<false, 4>);
+    k<<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below, chunk_len, P);
 }
 
 // ------------------------------------------------------------------ place
@@ -521,8 +529,7 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        if (below > 0) scan_kernel<true><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, below, len, P);
-        else scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len, P);
+        launch_scan<TR>(w, NB, below, len, P, st);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -568,7 +575,7 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
         return set_cuda_error(e);                       // non-finite count, tile-wait flag, checks
     const bool grad = !(flags & BSPLINE_INTERP_NO_GRAD);
     const bool ranked = launch_bin<TR, false, AT>(p, x, P, g, w, nullptr, nullptr, grid_for(P, 256), status, st);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, len, P);
+    launch_scan<TR>(w, NB, 0u, len, P, st);
     scatter_kernel<TR, AT><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, (double)p->N / p->L, p->order, g, w, (AT*)out_u, grad ? (AT*)out_grad : nullptr,
                                                              ranked, status);
     int rc = dispatch_order<CT, AT, TR>(p, coeffs, w, g, out_u, out_grad, grad, 0u);
@@ -624,7 +631,7 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCAN);
-        scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk, P);
+        launch_scan<TR>(w, NB, 0u, kChunk, P, st);
     }
     {
         StageTimer tm(p, BSPLINE_STAGE_SCATTER);
@@ -669,7 +676,7 @@ int run_sort_order(bspline_plan_s* p, const double* x, int64_t P, int* perm) {
         return set_cuda_error(e);
     const double scale = (double)p->N / p->L;
     const bool ranked = launch_bin<TR, false, float>(p, x, P, g, w, nullptr, nullptr, grid_for(P, 256), p->d_status, st);
-    scan_kernel<false><<<1, 1024, 0, st>>>(w.count, w.offset, w.cursor, w.chunk, w.item, NB, 0u, kChunk, P);
+    launch_scan<TR>(w, NB, 0u, kChunk, P, st);
     scatter_kernel<TR, float, false, true><<<grid_for(P, 256), 256, 0, st>>>(x, P, p->N, scale, p->order, g, w,
                                                                             (float*)nullptr, (float*)nullptr,
                                                                             ranked, p->d_status, perm);

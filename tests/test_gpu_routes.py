@@ -130,7 +130,7 @@ def test_sort_beside_the_transform_agrees_with_the_unsorted_call(B, dtype, split
     plan.close()
 
 
-@pytest.mark.parametrize("dtype,N", [("f64", 32), ("f64", 64), ("f32", 64), ("bf16", 128)])
+@pytest.mark.parametrize("dtype,N", [("f64", 32), ("f64", 64), ("f64", 128), ("f32", 64), ("bf16", 128)])
 def test_counting_by_runs_and_by_particles_agree(B, dtype, N):
     """Both sides of the rule that counts particles by runs in shared memory (12288 of them, 64 a brick): every
     particle is placed once, and its results are the same bits."""
@@ -155,4 +155,26 @@ def test_counting_by_runs_and_by_particles_agree(B, dtype, N):
     for u, grad in outs[1:]:
         assert torch.equal(torch.nan_to_num(u, 7.0), torch.nan_to_num(outs[0][0], 7.0))
         assert torch.equal(torch.nan_to_num(grad, 7.0), torch.nan_to_num(outs[0][1], 7.0))
+    plan.close()
+
+
+@pytest.mark.parametrize("N", [96, 192, 256])             # 288, 2304 and 5632 bricks: one to a thread, four, two tiles
+def test_scan_places_every_split(B, N):
+    """Bricks on both sides of the split and empty ones, some of them staged: every split gives the same bits."""
+    order, P = 4, 60000
+    plan = B.Plan(N, order, "f32")
+    g = torch.Generator(device="cuda").manual_seed(N)
+    coef = torch.randn((3, N, N, N), generator=g, device="cuda")
+    x = positions(P, N)
+    x[: P // 2] = torch.remainder(2.0 + 0.05 * L * torch.randn((P // 2, 3), generator=g, dtype=torch.float64, device="cuda"), L)
+    x[7, 0] = math.nan
+    plan.set_gather_split(0)
+    u0, g0 = plan.interp(coef, x)
+    assert plan.status() == 1
+    for split in (2, 16, 64, 1 << 30):
+        plan.set_gather_split(split)
+        u, grad = plan.interp(coef, x)
+        assert plan.status() == 1
+        for a, b in ((u, u0), (grad, g0)):
+            assert torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0)), split
     plan.close()
