@@ -489,7 +489,7 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    const unsigned len = item_particles(p->dtype, P, NB);
+    const unsigned len = item_particles(p->dtype, p->order, P, NB);
     const size_t need = carve<TR>(&w, nullptr, NB, P, shortest_item(p->dtype));
     int rc = p->pws.grow(need);
     if (rc) return rc;
@@ -566,7 +566,7 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    const unsigned len = item_particles(p->dtype, P, NB);
+    const unsigned len = item_particles(p->dtype, p->order, P, NB);
     carve<TR>(&w, ws, NB, P, shortest_item(p->dtype));
     cudaStream_t st = p->stream;
     cudaError_t e;

@@ -43,15 +43,23 @@ static_assert(sizeof(Rec<float>) == 32 && sizeof(Rec<double>) == 32, "one sector
 // Particles per gather work item: a brick with more particles is split into
 // several items, each staging the brick's tile, so no CTA serialises a clump.
 constexpr unsigned kChunk = 2048;
-// FP64 plans' evaluation: 512, and 42 when the bricks hold few particles (three components of 42 particles
-// are the 126 units of a 128-thread CTA; gather_fixed).
-constexpr unsigned kFixedLong = 512, kFixedShort = 42;
-inline unsigned item_particles(int dtype, int64_t P, unsigned NB) {
-    return dtype != BSPLINE_F64 ? kChunk : (P >= 256LL * NB ? kFixedLong : kFixedShort);
+// FP64 plans' evaluation: 512, or 42 (three components of 42 particles are the 126 units of a 128-thread CTA;
+// gather_fixed).  512 where the call has as many such items as fill the SMs, and the bricks hold so many particles that
+// staging and converting a tile for each 42 of them costs more than the long form's idle threads.  Measured, us a call
+// with items of 42 / 512, uniform particles, at 128^3 (4096 bricks), particles a brick in brackets: order 2 [8] 64 / 78,
+// [48] 127 / 116, [96] 199 / 176; order 4 [30] 149 / 196, [48] 224 / 216, [96] 352 / 258; order 6 [64] 476 / 487, [96] 666 / 530,
+// [256] 1487 / 1108; order 8 [64] 917 / 996, [96] 1293 / 1074; clustered, order 4 [64] 245 / 276, [128] 419 / 352.  At 32^3 (64
+// bricks), by the call's particles: order 4 65536 74 / 87, 131072 115 / 111, 200000 161 / 116; order 8 131072 372 / 307, 163840
+// 452 / 512, 262144 708 / 581.  At 64^3, order 6: 65536 129 / 135, 200000 299 / 273, clustered 129 / 195, 299 / 293.  Both give
+// the same bits.
+constexpr unsigned kFixedLong = 512, kFixedShort = 42, kFixedLongItems = 384;
+inline unsigned item_particles(int dtype, int order, int64_t P, unsigned NB) {
+    if (dtype != BSPLINE_F64) return kChunk;
+    const int64_t dense = order == 2 ? 32 : (order <= 4 ? 48 : 96);
+    return P >= (int64_t)kFixedLong * kFixedLongItems && P >= dense * NB ? kFixedLong : kFixedShort;
 }
-
 // The shortest items of a type: what the workspace holds places for, so that a call of fewer particles never needs a
-// larger one (131071 particles on 64^3 take items of 42, 131072 items of 512).
+// larger one because its items are of 42 instead of 512.
 constexpr unsigned shortest_item(int dtype) { return dtype == BSPLINE_F64 ? kFixedShort : kChunk; }
 
 template <typename TR> struct Ws {
@@ -1700,7 +1708,7 @@ int run_gather(bspline_plan_s* p, const void* coeffs, Ws<TR> w, BrickGrid g, voi
     const AT dscale = (AT)((double)p->N / p->L);
     int rc;
     if constexpr (sizeof(AT) == 8) {
-        const unsigned len = item_particles(p->dtype, w.P, NB);
+        const unsigned len = item_particles(p->dtype, ORD, w.P, NB);
         const bool whole = len == kFixedLong;
         auto k = whole ? (grad ? gather_fixed<ORD, TR, true, 3> : gather_fixed<ORD, TR, false, 3>)
                        : (grad ? gather_fixed<ORD, TR, true, 1> : gather_fixed<ORD, TR, false, 1>);

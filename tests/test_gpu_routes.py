@@ -34,11 +34,11 @@ def field(plan, seed):
 @pytest.mark.parametrize("N", [32, 64])
 def test_workspace_never_shrinks_with_more_particles(B, dtype, N):
     """A call of fewer particles after a larger one allocates nothing (it may be captured): across every rule
-    that depends on the count, such as the work items' length of FP64 plans (256 particles a brick)."""
+    that depends on the count, such as the work items' length of FP64 plans."""
     plan = B.Plan(N, 4, dtype)
     bricks = (N // 8) ** 3
-    counts = sorted({p + d for p in (1, 42, 512, 2048, 16 * bricks, 64 * bricks, 96 * bricks, 128 * bricks, 256 * bricks,
-                                     300000) for d in (-1, 0, 1) if p + d > 0})
+    counts = sorted({p + d for p in (1, 42, 512, 2048, 12288, 16 * bricks, 48 * bricks, 64 * bricks, 96 * bricks,
+                                     256 * bricks, 196608, 300000) for d in (-1, 0, 1) if p + d > 0})
     sizes = [plan.workspace_bytes(p) for p in counts]
     assert sizes == sorted(sizes)
     plan.close()
@@ -177,4 +177,24 @@ def test_scan_places_every_split(B, N):
         assert plan.status() == 1
         for a, b in ((u, u0), (grad, g0)):
             assert torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0)), split
+    plan.close()
+
+
+@pytest.mark.parametrize("order", [2, 3, 4, 5, 6, 7, 8])
+def test_long_and_short_items_of_fp64_plans_agree(B, order):
+    """200000 particles, 390 a brick, take items of 512, a tenth of them items of 42: the same bits, in a field some of
+    whose particles are left to FP64."""
+    N, P = 64, 200000
+    plan = B.Plan(N, order, "f64")
+    g = torch.Generator(device="cuda").manual_seed(order)
+    coef = torch.randn((3, N, N, N), generator=g, dtype=torch.float64, device="cuda")
+    coef[:, ::8, ::8, ::8] *= 100.0
+    x = positions(P, order)
+    x[1] = torch.tensor([0.0, L / 2, math.nextafter(L, 0.0)])
+    x[2, 0] = math.inf
+    u, grad = plan.interp(coef, x)
+    assert plan.status() == 1
+    u_few, grad_few = plan.interp(coef, x[: P // 10].contiguous())
+    for a, b in ((u, u_few), (grad, grad_few)):
+        assert torch.equal(torch.nan_to_num(a[: P // 10], 7.0), torch.nan_to_num(b, 7.0))
     plan.close()
