@@ -103,7 +103,7 @@ def rms(v):
 
 @pytest.mark.parametrize("kind", ["white", "outlier", "spike", "gaussian", "0.3", "1", "2"])
 @pytest.mark.parametrize("order", [3, 4, 6, 8])
-@pytest.mark.parametrize("P", [301, 2100])                # 8 bricks: short and long work items
+@pytest.mark.parametrize("P", [301, 2100])                # 8 bricks
 def test_evaluation_error_is_no_larger_than_fp64(B, kind, order, P):
     """Where the fixed form is taken its error is below FP64 arithmetic's, elsewhere it is FP64 arithmetic in
     another order of operations, which is what the factor 1.25 allows for."""
