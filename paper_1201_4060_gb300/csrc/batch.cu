@@ -147,7 +147,7 @@ int build_queue(bspline_batch_s* b, int by, unsigned chunk_len) {
     for (int i = 0; i < F; ++i) {
         gather_impl::Ws<float> w;
         off_ws[i] = off;
-        off = align256(off + gather_impl::carve<float>(&w, nullptr, grids[i].NB, b->P[i], chunk_len));
+        off = align256(off + gather_impl::carve<float>(&w, nullptr, grids[i].NB, b->P[i], true, chunk_len));
     }
     int rc = b->qbuf.grow(off);
     if (rc) return rc;
@@ -166,7 +166,7 @@ int build_queue(bspline_batch_s* b, int by, unsigned chunk_len) {
         d.scale = (double)p->N / p->L;
         d.dscale = (float)((double)p->N / p->L);
         d.bg = grids[i];
-        gather_impl::carve<float>(&d.w, base + off_ws[i], grids[i].NB, b->P[i], chunk_len);
+        gather_impl::carve<float>(&d.w, base + off_ws[i], grids[i].NB, b->P[i], true, chunk_len);
         d.w.count = reinterpret_cast<unsigned*>(base + off_counts) + cofs;   // the cleared block
         d.w.unsorted = d.w.count + grids[i].NB + 1;
         cofs += grids[i].NB + 2;

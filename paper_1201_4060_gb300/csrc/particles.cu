@@ -416,14 +416,13 @@ inline unsigned grid_for(long long P, int threads) {
 // 58.5 / 49.3; 4096 bricks, 64000 54.6 / 63.0, 256000 109.6 / 110.3, 10^6 310 / 293).  Never for sorted input: a warp's
 // particles share a brick or two, one atomic each, and nothing is placed afterwards (FP32, 64^3 in brick order,
 // histogram / warp: 2000 particles, order 4, 34.6 / 29.3 us a call; 50000 41.7 / 36.3; 10^6, order 2, 111 / 103).
-constexpr long long kHistLeast = 12288, kHistPerBrick = 64;   // particles in all, particles a brick
 template <typename TR, bool SORTED, typename OT>
 bool launch_bin(bspline_plan_s* p, const double* x, int64_t P, const BrickGrid& g, const Ws<TR>& w, OT* ou, OT* og,
                 unsigned grid, unsigned long long* status, cudaStream_t st) {
     const double scale = (double)p->N / p->L;
-    const unsigned run = (unsigned)std::min<long long>(8192, std::max<long long>(1024, (P / (2 * p->sms) + 255) / 256 * 256));
     if constexpr (!SORTED) {
-        if (g.NB <= std::max(run, 4096u) && P >= std::max(kHistLeast, kHistPerBrick * g.NB)) {
+        if (counts_by_runs(P, g.NB, p->sms)) {
+            const unsigned run = count_run_length(P, p->sms);
             const size_t sm = sizeof(unsigned) * (g.NB + 1 + run);
             auto k = bin_kernel<TR, false, true, OT>;
             if (set_smem(k, sm) == BSPLINE_OK) {
@@ -490,10 +489,11 @@ int run_interp(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P
     const unsigned NB = g.NB;
     Ws<TR> w;
     const unsigned len = item_particles(p->dtype, p->order, P, NB);
-    const size_t need = carve<TR>(&w, nullptr, NB, P, shortest_item(p->dtype));
+    const bool ranks = counts_by_runs(P, NB, p->sms);
+    const size_t need = carve<TR>(&w, nullptr, NB, P, ranks, shortest_item(p->dtype));
     int rc = p->pws.grow(need);
     if (rc) return rc;
-    carve<TR>(&w, p->pws.ptr, NB, P, shortest_item(p->dtype));
+    carve<TR>(&w, p->pws.ptr, NB, P, ranks, shortest_item(p->dtype));
     const cudaStream_t main_stream = p->stream;
     cudaStream_t st = sort_stream ? sort_stream : main_stream;
     p->stream = st;                                     // stage timers follow the sort's stream
@@ -567,7 +567,7 @@ int run_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, const
     const unsigned NB = g.NB;
     Ws<TR> w;
     const unsigned len = item_particles(p->dtype, p->order, P, NB);
-    carve<TR>(&w, ws, NB, P, shortest_item(p->dtype));
+    carve<TR>(&w, ws, NB, P, counts_by_runs(P, NB, p->sms), shortest_item(p->dtype));
     cudaStream_t st = p->stream;
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (NB + 2), st)) != cudaSuccess) return set_cuda_error(e);
@@ -608,10 +608,11 @@ int run_adjoint_particles(bspline_plan_s* p, const void* coeffs, const double* x
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    const size_t need = carve<TR>(&w, nullptr, NB, P);
+    const bool ranks = counts_by_runs(P, NB, p->sms);
+    const size_t need = carve<TR>(&w, nullptr, NB, P, ranks);
     int rc = p->pws.grow(need);
     if (rc) return rc;
-    carve<TR>(&w, p->pws.ptr, NB, P);
+    carve<TR>(&w, p->pws.ptr, NB, P, ranks);
     // FP32 types: the placement pass also copies each particle's cotangents to its sorted slot, which the
     // spread and the position gradients then read in order instead of gathering them from random indices
     float4* cot = nullptr;
@@ -665,10 +666,11 @@ int run_sort_order(bspline_plan_s* p, const double* x, int64_t P, int* perm) {
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
     Ws<TR> w;
-    const size_t need = carve<TR>(&w, nullptr, NB, P);
+    const bool ranks = counts_by_runs(P, NB, p->sms);
+    const size_t need = carve<TR>(&w, nullptr, NB, P, ranks);
     int rc = p->pws.grow(need);
     if (rc) return rc;
-    carve<TR>(&w, p->pws.ptr, NB, P);
+    carve<TR>(&w, p->pws.ptr, NB, P, ranks);
     cudaStream_t st = p->stream;
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (NB + 2), st)) != cudaSuccess) return set_cuda_error(e);
@@ -719,12 +721,13 @@ int launch_interp_ws(bspline_plan_s* p, void* ws, unsigned long long* status, co
 size_t interp_workspace_bytes(const bspline_plan_s* p, int64_t P) {
     const BrickGrid g = brick_grid(p->N, p->dtype, p->order);
     const unsigned NB = g.NB;
+    const bool ranks = counts_by_runs(P, NB, p->sms);
     if (p->dtype == BSPLINE_F64) {
         Ws<double> w;
-        return carve<double>(&w, nullptr, NB, P, shortest_item(p->dtype));
+        return carve<double>(&w, nullptr, NB, P, ranks, shortest_item(p->dtype));
     }
     Ws<float> w;
-    return carve<float>(&w, nullptr, NB, P, shortest_item(p->dtype));
+    return carve<float>(&w, nullptr, NB, P, ranks, shortest_item(p->dtype));
 }
 
 int launch_interp_split(bspline_plan_s* p, const void* coeffs, const double* x, int64_t P, void* out_u,

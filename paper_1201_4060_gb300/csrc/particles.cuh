@@ -62,13 +62,23 @@ inline unsigned item_particles(int dtype, int order, int64_t P, unsigned NB) {
 // larger one because its items are of 42 instead of 512.
 constexpr unsigned shortest_item(int dtype) { return dtype == BSPLINE_F64 ? kFixedShort : kChunk; }
 
+// Particles of a run of the count pass, and whether it goes by runs, which give each particle its place within its
+// brick (launch_bin says why).  Both grow with P: a call of fewer particles needs no larger workspace.
+constexpr int64_t kHistLeast = 12288, kHistPerBrick = 64;     // particles in all, particles a brick
+inline unsigned count_run_length(int64_t P, int sms) {
+    return (unsigned)std::min<int64_t>(8192, std::max<int64_t>(1024, (P / (2 * sms) + 255) / 256 * 256));
+}
+inline bool counts_by_runs(int64_t P, unsigned NB, int sms) {
+    return NB <= std::max(count_run_length(P, sms), 4096u) && P >= std::max<int64_t>(kHistLeast, kHistPerBrick * NB);
+}
+
 template <typename TR> struct Ws {
     unsigned* count;    // [NB + 2]  particles per brick; slot NB = invalid positions; NB + 1 = *unsorted
     unsigned* unsorted; // nonzero if positions passed as sorted were not in brick order (count pass)
     unsigned* offset;   // [NB + 3]  start of each brick's sorted segment; [NB] end of the valid
                         //           particles, [NB + 1] end of all, [NB + 2] start of the sparse range
     unsigned* cursor;   // [NB + 1]  next free sorted slot of each brick (starts at offset), without ranks
-    unsigned* rank;     // [P]       each particle's place within its brick (count pass by histograms)
+    unsigned* rank;     // [P]       each particle's place within its brick (count pass by runs; else none)
     unsigned* chunk;    // [NB + 1]  exclusive prefix sum of ceil(count / chunk_len): first work item of a brick
     unsigned* item;     // [NB + ceil(P / shortest)]  brick of each work item (the first chunk[NB] are set)
     long long P;        // particles
@@ -77,7 +87,7 @@ template <typename TR> struct Ws {
 
 constexpr size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
-template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t P, unsigned shortest = kChunk) {
+template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t P, bool ranks, unsigned shortest = kChunk) {
     size_t off = 0;
     auto take = [&](size_t bytes) {
         void* ptr = base ? (void*)((char*)base + off) : nullptr;
@@ -89,7 +99,7 @@ template <typename TR> size_t carve(Ws<TR>* w, void* base, unsigned NB, int64_t 
     w->unsorted = base ? w->count + NB + 1 : nullptr;
     w->offset = (unsigned*)take(sizeof(unsigned) * (NB + 3));
     w->cursor = (unsigned*)take(sizeof(unsigned) * (NB + 1));
-    w->rank = (unsigned*)take(sizeof(unsigned) * P);
+    w->rank = (unsigned*)take(ranks ? sizeof(unsigned) * P : 0);
     w->chunk = (unsigned*)take(sizeof(unsigned) * (NB + 1));
     w->item = (unsigned*)take(sizeof(unsigned) * (NB + (P + shortest - 1) / shortest));
     w->s_rec = (Rec<TR>*)take(sizeof(Rec<TR>) * P);

@@ -44,6 +44,19 @@ def test_workspace_never_shrinks_with_more_particles(B, dtype, N):
     plan.close()
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_workspace_holds_ranks_only_where_the_count_draws_them(B, dtype):
+    """4 bytes a particle, beside the record's 32 and an FP64 item's 4 for 42, only from 64 particles a brick on."""
+    plan = B.Plan(64, 4, dtype)
+    bricks = 512 if dtype == "f64" else 96
+    edge = max(12288, 64 * bricks)
+    per_particle = 32 + (4 / 42 if dtype == "f64" else 4 / 2048)
+    fixed = plan.workspace_bytes(1)
+    assert plan.workspace_bytes(edge - 1) <= fixed + per_particle * edge + 4096
+    assert plan.workspace_bytes(edge) >= fixed + (per_particle + 4) * edge - 4096
+    plan.close()
+
+
 def key(N, order, P, route):
     return (f"{torch.cuda.get_device_properties(0).name}|N{N}|o{order}|f32|p2^{max(P - 1, 1).bit_length()}"
             + (f"|{route}" if route else ""))
