@@ -412,8 +412,8 @@ inline unsigned grid_for(long long P, int threads) {
 // warps queued for).  Else an atomic a particle and pass: at 512^3 (44032 bricks, 2^24 particles) places
 // returned by the count's atomics made the step 1.5 % slower; at 5632 bricks and 10^6 particles the runs
 // (3328) gain nothing.  Few particles do not repay the zeroing and flushing of the bins (FP64 u at order 2, atomics /
-// histogram, us a call: 64 bricks, 4000 particles 30.2 / 33.1, 16000 37.2 / 35.5; 512 bricks, 16000 36.8 / 38.6, 64000
-// 58.5 / 49.3; 4096 bricks, 64000 54.6 / 63.0, 256000 109.6 / 110.3, 10^6 310 / 293).  Never for sorted input: a warp's
+// histogram, us a call: 64 bricks, 4000 particles 30.2 / 33.1, 16000 37.2 / 35.5, and 10^4 beside the transform at order 4
+// 45.9 / 44.2; 512 bricks, 16000 36.8 / 38.6, 64000 58.5 / 49.3; 4096 bricks, 64000 54.6 / 63.0, 256000 109.6 / 110.3, 10^6 310 / 293).  Never for sorted input: a warp's
 // particles share a brick or two, one atomic each, and nothing is placed afterwards (FP32, 64^3 in brick order,
 // histogram / warp: 2000 particles, order 4, 34.6 / 29.3 us a call; 50000 41.7 / 36.3; 10^6, order 2, 111 / 103).
 template <typename TR, bool SORTED, typename OT>

@@ -64,7 +64,7 @@ constexpr unsigned shortest_item(int dtype) { return dtype == BSPLINE_F64 ? kFix
 
 // Particles of a run of the count pass, and whether it goes by runs, which give each particle its place within its
 // brick (launch_bin says why).  Both grow with P: a call of fewer particles needs no larger workspace.
-constexpr int64_t kHistLeast = 12288, kHistPerBrick = 64;     // particles in all, particles a brick
+constexpr int64_t kHistLeast = 8192, kHistPerBrick = 64;     // particles in all, particles a brick
 inline unsigned count_run_length(int64_t P, int sms) {
     return (unsigned)std::min<int64_t>(8192, std::max<int64_t>(1024, (P / (2 * sms) + 255) / 256 * 256));
 }

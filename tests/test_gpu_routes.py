@@ -37,7 +37,7 @@ def test_workspace_never_shrinks_with_more_particles(B, dtype, N):
     that depends on the count, such as the work items' length of FP64 plans."""
     plan = B.Plan(N, 4, dtype)
     bricks = (N // 8) ** 3
-    counts = sorted({p + d for p in (1, 42, 512, 2048, 12288, 16 * bricks, 48 * bricks, 64 * bricks, 96 * bricks,
+    counts = sorted({p + d for p in (1, 42, 512, 2048, 8192, 16 * bricks, 48 * bricks, 64 * bricks, 96 * bricks,
                                      256 * bricks, 196608, 300000) for d in (-1, 0, 1) if p + d > 0})
     sizes = [plan.workspace_bytes(p) for p in counts]
     assert sizes == sorted(sizes)
@@ -49,7 +49,7 @@ def test_workspace_holds_ranks_only_where_the_count_draws_them(B, dtype):
     """4 bytes a particle, beside the record's 32 and an FP64 item's 4 for 42, only from 64 particles a brick on."""
     plan = B.Plan(64, 4, dtype)
     bricks = 512 if dtype == "f64" else 96
-    edge = max(12288, 64 * bricks)
+    edge = max(8192, 64 * bricks)
     per_particle = 32 + (4 / 42 if dtype == "f64" else 4 / 2048)
     fixed = plan.workspace_bytes(1)
     assert plan.workspace_bytes(edge - 1) <= fixed + per_particle * edge + 4096
@@ -145,13 +145,13 @@ def test_sort_beside_the_transform_agrees_with_the_unsorted_call(B, dtype, split
 
 @pytest.mark.parametrize("dtype,N", [("f64", 32), ("f64", 64), ("f64", 128), ("f32", 64), ("bf16", 128)])
 def test_counting_by_runs_and_by_particles_agree(B, dtype, N):
-    """Both sides of the rule that counts particles by runs in shared memory (12288 of them, 64 a brick): every
+    """Both sides of the rule that counts particles by runs in shared memory (8192 of them, 64 a brick): every
     particle is placed once, and its results are the same bits."""
     order = 3
     plan = B.Plan(N, order, dtype)
     plan.set_gather_split(0)
     bricks = (N // 8) ** 3 if dtype == "f64" else (N // 16) ** 2 * -(-N // 12)
-    edge = max(12288, 64 * bricks)
+    edge = max(8192, 64 * bricks)
     g = torch.Generator(device="cuda").manual_seed(N)
     real = torch.float64 if dtype == "f64" else torch.float32
     coef = torch.randn((3, N, N, N), generator=g, dtype=real, device="cuda").to(plan.coef_dtype)
