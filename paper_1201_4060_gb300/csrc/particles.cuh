@@ -910,16 +910,6 @@ template <int n, int k = 2> __device__ __forceinline__ void weights_f64(double t
         }
     }
 }
-template <bool GRAD>
-__device__ __forceinline__ void store_f64(double u, double gx, double gy, double gz, double dscale,
-                                          double* __restrict__ out_u, double* __restrict__ out_grad) {
-    *out_u = u;
-    if (GRAD) {
-        out_grad[0] = gx * dscale;
-        out_grad[1] = gy * dscale;
-        out_grad[2] = gz * dscale;
-    }
-}
 template <int ORD, bool GRAD>
 __device__ __noinline__ void eval_f64_thread(const double* __restrict__ comp, int N, unsigned cell, double tx,
                                              double ty, double tz, double dscale, double* __restrict__ out_u,
@@ -959,7 +949,12 @@ __device__ __noinline__ void eval_f64_thread(const double* __restrict__ comp, in
             gz = fma(wx[jx], y01, gz);
         }
     }
-    store_f64<GRAD>(u, gx, gy, gz, dscale, out_u, out_grad);
+    *out_u = u;
+    if (GRAD) {
+        out_grad[0] = gx * dscale;
+        out_grad[1] = gy * dscale;
+        out_grad[2] = gz * dscale;
+    }
 }
 
 // The recurrence with lane (axis, m) holding v[m]: after step k < n, M_k(t + m); then the node's two weights.
@@ -973,18 +968,20 @@ template <int n, int k = 2> __device__ __forceinline__ void weights_f64_warp(dou
         *dw = v - b;
     }
 }
+// Sums by lane, each in the order of eval_f64_thread: along z, chain 2 line + s (s = 0: w, 1: w'); along y, lane
+// s ORD + jx (s = 0: Y00, 1: Y10, 2: Y01); along x, lanes 0 to 3 (u and the three derivatives).
 template <int ORD, bool GRAD>
 __device__ __noinline__ void eval_f64_warp(const double* __restrict__ comp, int N, unsigned cell, double tx,
                                            double ty, double tz, double dscale, double* __restrict__ out_u,
                                            double* __restrict__ out_grad) {
     constexpr unsigned kAll = 0xffffffffu;
-    constexpr int R = (ORD * ORD + 31) / 32;             // lines of a lane
+    constexpr int C = 2 * ORD * ORD, R = (C + 31) / 32;  // chains, and those of a lane
     const int lane = threadIdx.x & 31;
     const int ax = (int)(cell >> (2 * kAnchorBits)), ay = (int)((cell >> kAnchorBits) & 1023u), az = (int)(cell & 1023u);
     double v[R][ORD];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int l = min(lane + 32 * r, ORD * ORD - 1), jx = l / ORD, jy = l % ORD;
+        const int l = min(lane + 32 * r, C - 1) >> 1, jx = l / ORD, jy = l % ORD;
         const double* line = comp + ((size_t)wrap_index(ax + jx, N) * N + wrap_index(ay + jy, N)) * N;
 #pragma unroll
         for (int jz = 0; jz < ORD; ++jz) v[r][jz] = line[wrap_index(az + jz, N)];
@@ -992,51 +989,36 @@ __device__ __noinline__ void eval_f64_warp(const double* __restrict__ comp, int 
     double w, dw;                                        // lane a ORD + m: node ORD - 1 - m of axis a
     const int a = lane / ORD;
     weights_f64_warp<ORD>(a == 0 ? tx : (a == 1 ? ty : tz), lane % ORD, lane % ORD == 0 ? 1.0 : 0.0, &w, &dw);
-    double z0[R], z1[R];
+    const auto weight = [&](int axis, int j, bool derivative) {
+        const double wj = __shfl_sync(kAll, w, (axis + 1) * ORD - 1 - j), dj = __shfl_sync(kAll, dw, (axis + 1) * ORD - 1 - j);
+        return derivative ? dj : wj;
+    };
+    double z[R], y = 0, x = 0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) z0[r] = z1[r] = 0.0;
+    for (int r = 0; r < R; ++r) z[r] = 0.0;
 #pragma unroll
     for (int jz = 0; jz < ORD; ++jz) {
-        const double wj = __shfl_sync(kAll, w, 3 * ORD - 1 - jz), dj = __shfl_sync(kAll, dw, 3 * ORD - 1 - jz);
+        const double wj = weight(2, jz, lane & 1);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            z0[r] = fma(wj, v[r][jz], z0[r]);
-            if (GRAD) z1[r] = fma(dj, v[r][jz], z1[r]);
-        }
+        for (int r = 0; r < R; ++r) z[r] = fma(wj, v[r][jz], z[r]);
     }
-    double y00 = 0, y10 = 0, y01 = 0;                    // lane jx: the x-row's
+    const int sy = min(lane / ORD, 2), jx0 = lane % ORD;
 #pragma unroll
     for (int jy = 0; jy < ORD; ++jy) {
-        const int l = min(lane, ORD - 1) * ORD + jy;
-        double a0 = 0, a1 = 0;
+        const int chain = 2 * (jx0 * ORD + jy) + (sy == 2 ? 1 : 0);
+        double b = 0;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const double b0 = __shfl_sync(kAll, z0[r], l & 31), b1 = __shfl_sync(kAll, z1[r], l & 31);
-            if ((l >> 5) == r) {
-                a0 = b0;
-                a1 = b1;
-            }
+            const double br = __shfl_sync(kAll, z[r], chain & 31);
+            if ((chain >> 5) == r) b = br;
         }
-        const double wj = __shfl_sync(kAll, w, 2 * ORD - 1 - jy), dj = __shfl_sync(kAll, dw, 2 * ORD - 1 - jy);
-        y00 = fma(wj, a0, y00);
-        if (GRAD) {
-            y10 = fma(dj, a0, y10);
-            y01 = fma(wj, a1, y01);
-        }
+        y = fma(weight(1, jy, sy == 1), b, y);
     }
-    double u = 0, gx = 0, gy = 0, gz = 0;
+    const int sx = lane < 2 ? 0 : min(lane - 1, 2);      // lanes 0, 1: Y00, 2: Y10, 3: Y01
 #pragma unroll
-    for (int jx = 0; jx < ORD; ++jx) {
-        const double wj = __shfl_sync(kAll, w, ORD - 1 - jx), dj = __shfl_sync(kAll, dw, ORD - 1 - jx);
-        const double b00 = __shfl_sync(kAll, y00, jx);
-        u = fma(wj, b00, u);
-        if (GRAD) {
-            gx = fma(dj, b00, gx);
-            gy = fma(wj, __shfl_sync(kAll, y10, jx), gy);
-            gz = fma(wj, __shfl_sync(kAll, y01, jx), gz);
-        }
-    }
-    if (lane == 0) store_f64<GRAD>(u, gx, gy, gz, dscale, out_u, out_grad);
+    for (int jx = 0; jx < ORD; ++jx) x = fma(weight(0, jx, lane == 1), __shfl_sync(kAll, y, sx * ORD + jx), x);
+    if (lane == 0) *out_u = x;
+    else if (GRAD && lane < 4) out_grad[lane - 1] = x * dscale;
 }
 
 // FP64 plans: one CTA per work item, the brick's coefficients staged and turned into 60-bit fixed point
@@ -1262,8 +1244,10 @@ gather_fixed(const double* __restrict__ coef, int N, BrickGrid bg, Ws<TR> w, uns
             evaluate(rc, i, 0, [&](int j) { return ws[j * T + threadIdx.x]; }, wy, dwy, wz, dwz);
         }
     }
-    // those left over, in FP64: few of them a warp each, many a thread each (a warp's form takes 54 to 130 FP64
-    // instructions a pair, a thread's 340 to 1700 for up to 32 pairs)
+    // those left over, in FP64: few of them a warp each, many a thread each (a warp's form takes 30 to 80 FP64
+    // instructions a pair, a thread's 340 to 1700 for up to 32 pairs).  10^4 particles on 32^3 in one product of modes (4 to
+    // 8 % left over, gathered in the bricks of its nodal lines), up to 8 / 12 / 20 pairs a warp: order 4 55 / 61 / 61 us,
+    // order 8 152 / 148 / 142; a narrow Gaussian, nearly all left over, order 4 63 / 67 / 80, order 8 180 / 179 / 211
     __syncthreads();
     const unsigned left = s_left;
     const bool by_warp = left <= 8 * (T / 32);
