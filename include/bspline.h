@@ -52,8 +52,11 @@ extern "C" {
 typedef struct bspline_plan_s* bspline_plan_t;
 
 /* Coefficient storage type.  F64: FP64 data; the transform and the evaluation
- * compute in 60-bit fixed point where the values allow it (every result at
- * least as exact as FP64 arithmetic) and in FP64 elsewhere.  F32: FP32 transform,
+ * compute in 60-bit fixed point where its rounding is below that of FP64
+ * arithmetic on the same values, and in FP64 elsewhere.  The error of u is a
+ * multiple of 2^-53 sum w |a| over the particle's stencil (node weights w,
+ * coefficients a), however steep the coefficients are; that of the
+ * coefficients, line by line of the transform, of the line's rms.  F32: FP32 transform,
  * FP32 coefficients, FP32 weights and accumulation.  BF16: FP32 transform,
  * coefficients rounded to bfloat16 on store, FP32 weights and accumulation.
  * Position-to-cell index and local offset are computed in FP64 for all. */

@@ -16,8 +16,8 @@
 // Lines whose largest magnitude is not in 2^[-895, 977], or that hold a NaN or an infinity, make their tile
 // take the FP64 stages (the caller).  p depends on the line's values alone.
 //
-// Bound: integer issue (the ALU pipe half busy; 64-bit adds and the limbs' shifts).  Measured at 256^3 FP64:
-// X pass 1.31 -> 0.33 ms, ky/kz pass 2.70 -> 0.91 ms; coefficients 4.5e-16 -> 4.1e-16 off 64-bit references.
+// Bound: integer issue (64-bit adds and the limbs' shifts; the ky/kz pass also by missing instructions).  Measured at
+// 256^3, FP64 stages / one scale a line / block floating point: X pass 1.31 / 0.33 / 0.35 ms, ky/kz pass 2.70 / 0.90 / 0.94.
 #pragma once
 #include "fft_core.cuh"
 #include "fixed.cuh"

@@ -1033,8 +1033,8 @@ __device__ __noinline__ void eval_f64_warp(const double* __restrict__ comp, int 
 // fixed form where sum w |a| is at least 2^53 units (fixed::contract gives a lower estimate); the others, and every
 // particle of a component whose tile holds a NaN or an infinity or nothing above 2^-895, are evaluated in FP64
 // from global memory (eval_f64_thread, eval_f64_warp): the low flanks of steep or localised fields, one particle
-// in 10^4 or fewer of a turbulent one, 1 % in a single Fourier mode (its nodal planes).  That choice depends on the
-// coefficients and the position alone, so every route to the evaluation gives the same bits.
+// in 10^4 or fewer of a turbulent one, 1 to 8 % of a product of Fourier modes (where its nodal planes meet).  That choice
+// depends on the coefficients and the position alone, so every route to the evaluation gives the same bits.
 // Order 2 stays in FP64: with eight nodes a component the conversion costs more than it saves (256^3, 10^6
 // particles, a call 0.48 ms in FP64, 0.50 ms in fixed point).
 // NC = 3: a thread takes a particle's components in turn; NC = 1 (items of up to 42 particles): a thread
